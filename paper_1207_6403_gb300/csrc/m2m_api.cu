@@ -125,6 +125,8 @@ struct m2m_ctx {
     long long wait_ns = 2000000000ll;      // limit of one grid-barrier wait
     int test_stall = 0;              // test only: the next launch's block 0 skips its first arrival
     long long test_wait_ns = 0;      //   and its barrier waits are limited to this
+    void *d_vm = nullptr;            // velocity moments: sums and shell edges
+    size_t vm_bytes = 0;
     // particle shards (m2m_shard_*): this context holds one shard of a model
     bool shard = false;
     bool shard_push = false;         // the last shard scatter pushed
@@ -615,7 +617,7 @@ void free_all(m2m_ctx *c) {
                     c->d_last, c->d_err, c->d_mm_slots, c->d_cell_ids, c->d_cell_acc, c->d_cell_cnt,
                     c->d_cell_mean, c->d_cell_cache, c->d_y_acc, c->d_sh_e2, c->d_sh_rn, c->d_sh_irn,
                     c->d_sh_tab, c->d_sh_rnd, c->d_sh_sum, c->d_facc, c->d_lnwhat, c->d_lut, c->d_pmap, c->d_psf,
-                    c->d_bar, c->d_st2, c->d_chi2};
+                    c->d_bar, c->d_st2, c->d_chi2, c->d_vm};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -1310,21 +1312,38 @@ int m2m_velocity_moments(m2m_ctx *ctx, const double *r2_edges, int32_t nshell, d
             return set_err(ctx, M2M_ERR_ARG, "edges must be strictly increasing");
     int rc = finish_update(ctx);
     if (rc) return rc;
-    const size_t eb = 8 * (size_t)(nshell + 1), ob = 32 * (size_t)nshell;
-    void *d = nullptr;
-    CU(cudaMallocAsync(&d, eb + ob, ctx->st));
-    double *de = (double *)d, *dout = de + (nshell + 1);
-    cudaError_t e = cudaMemcpyAsync(de, r2_edges, eb, cudaMemcpyHostToDevice, ctx->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dout, 0, ob, ctx->st);
+    // the edges in the state precision and the cleared sums in one upload, to a
+    // buffer the context keeps (an allocation per call cost 200 us: the pool
+    // gave its memory back at every synchronisation)
+    const bool f32 = ctx->prec == M2M_FP32C;
+    const size_t ob = 32 * (size_t)nshell, eb = (f32 ? 4 : 8) * (size_t)(nshell + 1);
+    if (ctx->vm_bytes < ob + eb) {
+        CU(cudaStreamSynchronize(ctx->st));
+        if (ctx->d_vm) cudaFree(ctx->d_vm);
+        ctx->d_vm = nullptr;
+        ctx->vm_bytes = 0;
+        CU(cudaMalloc(&ctx->d_vm, ob + eb));
+        ctx->vm_bytes = ob + eb;
+    }
+    std::vector<unsigned char> up(ob + eb, 0);
+    for (int k = 0; k <= nshell; ++k) {
+        if (f32) ((float *)(up.data() + ob))[k] = ceil_float(r2_edges[k]);
+        else ((double *)(up.data() + ob))[k] = r2_edges[k];
+    }
+    double *dout = (double *)ctx->d_vm;
+    void *de = (unsigned char *)ctx->d_vm + ob;
+    cudaError_t e = cudaMemcpyAsync(dout, up.data(), ob + eb, cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess) {
-        const size_t sm = ob + eb;
+        const int copies = vmoments_copies(nshell);
+        const size_t sm = ob * copies + eb;
         int g = ctx->nsm * 4;
         long long need = (ctx->n + 255) / 256;
         if (g > need) g = (int)need;
-        if (ctx->prec == M2M_FP32C)
+        if (f32)
             k_vmoments<float><<<g, 256, sm, ctx->st>>>((const float *)ctx->x, (const float *)ctx->y, (const float *)ctx->z,
                                                         (const float *)ctx->vx, (const float *)ctx->vy,
-                                                        (const float *)ctx->vz, ctx->w, ctx->n, de, nshell, dout);
+                                                        (const float *)ctx->vz, ctx->w, ctx->n, (const float *)de,
+                                                        nshell, copies, dout);
         else
             k_vmoments<double><<<g, 256, sm, ctx->st>>>((const double *)ctx->x, (const double *)ctx->y,
                                                          (const double *)ctx->z, (const double *)ctx->vx,
