@@ -81,6 +81,7 @@ struct PassArgs {
     void *slots;                            // FP64: [grid][nobs] double per-block sums
     unsigned long long *y_acc;              // FP32C: [nobs] int64 fixed-point totals
     int fx_atomic;                          // FP32C: flush to y_acc with atomics (else slots)
+    int hrep;                               // FP32C: copies of the block histogram's lower parts (see hist_copies)
     int fx_shift;                           // fixed point: value * 2^fx_shift
     int cell_shift;                         // FP32C prior-cell sums: weight * 2^cell_shift
     double *stat_slots;                     // [grid][2]: S, sum w
@@ -1134,7 +1135,8 @@ __device__ __forceinline__ void gh_red_stream(float vlos, const float4 *r, float
     fx_red_fast(Lo, Mid, b + 4, Wg * fmaf(m2, fmaf(K4, m2, c.w), (c.w * c.w) * C4));
 }
 
-__device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, float v, float fscale, int sh,
+// (b: index of the lower parts, h: of the high part)
+__device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, int hb, float v, float fscale, int sh,
                                        bool &ovf) {
     const float S = v * fscale;
     int h, l;
@@ -1146,14 +1148,14 @@ __device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, float 
         const int A = (h + 32768) >> 16;
         atomicAdd(Lo + b, l);
         atomicAdd(Mid + b, h - (A << 16));
-        if (A) atomicAdd(Hi + b, A);
+        if (A) atomicAdd(Hi + hb, A);
     } else {
         const long long q = f2fixed(v, sh, ovf);
         const long long hh = (q + 32768) >> 16;
         const long long A = (hh + 32768) >> 16;
         atomicAdd(Lo + b, (int)(q - (hh << 16)));
         atomicAdd(Mid + b, (int)(hh - (A << 16)));
-        atomicAdd(Hi + b, (int)A);
+        atomicAdd(Hi + hb, (int)A);
     }
 }
 

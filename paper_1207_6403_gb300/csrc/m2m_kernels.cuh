@@ -296,10 +296,10 @@ __device__ __forceinline__ void stage(T *dst, const T *src, int n, int tid, int 
 // rounding as the carve-up at the top of pass_body, without the pipeline's
 // stage buffers).  sh_len: SH node-table values staged when the pass pushes.
 inline size_t pass_smem_bytes(bool f32, int layout, int flags, int nobs, int edge_len, int gh_len, int sh_len,
-                              int nE, int nL, int ncells, int pmap_len = 0) {
+                              int nE, int nL, int ncells, int pmap_len = 0, int hrep = 1) {
     const size_t rs = f32 ? 4 : 8;
     size_t b = 0;
-    if (flags & F_SCAT) b += f32 ? 12 * (size_t)((nobs + 3) & ~3) : 8 * (size_t)((nobs + 1) & ~1);
+    if (flags & F_SCAT) b += f32 ? (4 + 8 * (size_t)hrep) * ((nobs + 3) & ~3) : 8 * (size_t)((nobs + 1) & ~1);
     if (flags & F_UPD) b += rs * (size_t)((nobs + 3) & ~3);
     b += rs * (size_t)((edge_len + 3) & ~3);
     b += 2 * rs * (size_t)((edge_len + 1) & ~1);                     // edge pairs
@@ -316,9 +316,21 @@ inline size_t pass_smem_bytes(bool f32, int layout, int flags, int nobs, int edg
     return b;
 }
 
+// Copies of the FP32C histogram's lower parts a block keeps (the layouts with
+// few observables): lane l of every warp adds to copy l mod copies.  With 32
+// copies the 32 lanes of an atomic hit 32 different banks whatever their
+// cells, so it is one shared-memory wavefront; with one copy, lanes that
+// share a cell or a bank queue behind each other.  The moments of copy r of
+// cell c (first observable b, nmom moments) are at b * copies + r * nmom + m:
+// 1 and 5 moments are both odd strides, so copies differ in their bank for
+// every moment.  The copies are summed when the histogram is flushed
+// (fx_totals); integer sums, so the totals do not depend on the copies.
+template <int L> constexpr bool hist_copied = L == 2 || L == 3;
+
 template <class R>
 struct PassSmem {
     int *hL, *hM, *hH;       // FP32C histogram: V = H * 2^32 + M * 2^16 + L per bin (exact fixed point)
+    int hrep, hlane;         //   copies of L and M, and this lane's copy (see hist_copies)
     double *h_d;             // FP64 histogram
     const R *coef, *edges, *gh;
     const Pair<R> *epair;    // (e[k], e[k+1]) for every edge-table index k
@@ -460,11 +472,74 @@ struct ThreadAcc {
     bool ovf, bad;
 };
 
-__device__ __forceinline__ void hist_add(const PassSmem<float> &S, int b, float v, float fs, int sh, ThreadAcc &t) {
-    fx_red(S.hL, S.hM, S.hH, b, v, fs, sh, t.ovf);
+// Index of moment 0 of this lane's copy of the cell whose first observable
+// is b.
+template <int L>
+__device__ __forceinline__ int hist_at(const PassSmem<float> &S, int b, int nmom) {
+    if constexpr (hist_copied<L>) return b * S.hrep + S.hlane * nmom;
+    return b;
 }
-__device__ __forceinline__ void hist_add(const PassSmem<double> &S, int b, double v, float, int, ThreadAcc &) {
-    atomicAdd(S.h_d + b, v);
+
+// Adds v to moment m of the cell whose first observable is b (i: hist_at).
+__device__ __forceinline__ void hist_add(const PassSmem<float> &S, int i, int b, int m, float v, float fs, int sh,
+                                         ThreadAcc &t) {
+    fx_red(S.hL, S.hM, S.hH, i + m, b + m, v, fs, sh, t.ovf);
+}
+__device__ __forceinline__ void hist_add(const PassSmem<double> &S, int, int b, int m, double v, float, int,
+                                         ThreadAcc &) {
+    atomicAdd(S.h_d + b + m, v);
+}
+template <int L>
+__device__ __forceinline__ int hist_at(const PassSmem<double> &, int b, int) { return b; }
+
+// The exact totals H * 2^32 + M * 2^16 + L of the block's FP32C histogram,
+// f(j, total) for every observable j, by `nw` warps of which this is `w`
+// (whole warps, after a barrier); clear: the histogram is zeroed for the next
+// segment.  With copies, two lanes share an observable, each summing half of
+// its copies; lane pair o starts at the copy that puts moment m on bank o
+// (13 = 1/5 mod 32), so that a warp's 32 loads hit 32 banks.
+template <int L, class F>
+__device__ __forceinline__ void fx_totals(const PassArgs &a, const PassSmem<float> &S, int w, int nw, bool clear,
+                                          F &&f) {
+    const int lane = threadIdx.x & 31, nobs = a.nobs;
+    auto total = [&](int k, int lo, int mid) {
+        return (long long)(((unsigned long long)(long long)S.hH[k] << 32) +
+                           ((unsigned long long)(long long)mid << 16) + (unsigned long long)(long long)lo);
+    };
+    if (!hist_copied<L> || S.hrep == 1) {
+        for (int k = 32 * w + lane; k < nobs; k += 32 * nw) {
+            const long long v = total(k, S.hL[k], S.hM[k]);
+            if (clear) { S.hL[k] = 0; S.hM[k] = 0; S.hH[k] = 0; }
+            f(k, v);
+        }
+        return;
+    }
+    const int R = S.hrep, o = lane >> 1;
+    for (int k0 = 16 * w; k0 < nobs; k0 += 16 * nw) {
+        const int k = k0 + o;
+        int lo = 0, mid = 0;
+        if (k < nobs) {
+            int off = 0, nmom = 1;
+            for (int q = 0; q < a.nsets; ++q)
+                if (k >= a.sets[q].obs_off) { off = a.sets[q].obs_off; nmom = a.sets[q].nmom; }
+            const int m = nmom == 5 ? (k - off) % 5 : 0, base = (k - m) * R + m;
+            const int s = (nmom == 5 ? 13 * (o - m) : o) + (lane & 1) * (R >> 1);
+#pragma unroll 4
+            for (int q = 0; q < (R >> 1); ++q) {
+                const int i = base + ((s + q) & (R - 1)) * nmom;
+                lo += S.hL[i];
+                mid += S.hM[i];
+                if (clear) { S.hL[i] = 0; S.hM[i] = 0; }
+            }
+        }
+        lo += __shfl_xor_sync(0xffffffffu, lo, 1);
+        mid += __shfl_xor_sync(0xffffffffu, mid, 1);
+        if (k < nobs && !(lane & 1)) {
+            const long long v = total(k, lo, mid);
+            if (clear) S.hH[k] = 0;
+            f(k, v);
+        }
+    }
 }
 
 template <class R, int L>
@@ -480,16 +555,16 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
             if (s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);
             int c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
             if (c < 0) continue;
-            int b = s.obs_off + c * s.nmom;
+            const int b = s.obs_off + c * s.nmom, h = hist_at<L>(S, b, s.nmom);
             if (s.quant == M2M_Q_MASS) {
-                hist_add(S, b, wv, fs, sh, ovf);
+                hist_add(S, h, b, 0, wv, fs, sh, ovf);
             } else if (s.quant == M2M_Q_VLOS2) {
-                hist_add(S, b, wv * (vlos * vlos), fs, sh, ovf);
+                hist_add(S, h, b, 0, wv * (vlos * vlos), fs, sh, ovf);
             } else {
                 R u[5];
                 gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
 #pragma unroll
-                for (int m = 0; m < 5; ++m) hist_add(S, b + m, wv * u[m], fs, sh, ovf);
+                for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
             }
         }
     } else {
@@ -509,15 +584,16 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
             if (c >= 0 && wv != R(0)) {
                 if constexpr (q == M2M_Q_MASS || q == M2M_Q_VLOS2) {
                     const R v = q == M2M_Q_MASS ? wv : wv * (vlos * vlos);
+                    const int b = s.obs_off + c, h = hist_at<L>(S, b, 1);
                     if constexpr (sizeof(R) == 4) {
                         const float Sv = v * fs;
-                        if (fabsf(Sv) < FX_FAST) fx_red_fast(S.hL, S.hM, s.obs_off + c, Sv);
-                        else hist_add(S, s.obs_off + c, v, fs, sh, ovf);
+                        if (fabsf(Sv) < FX_FAST) fx_red_fast(S.hL, S.hM, h, Sv);
+                        else hist_add(S, h, b, 0, v, fs, sh, ovf);
                     } else {
-                        hist_add(S, s.obs_off + c, v, fs, sh, ovf);
+                        hist_add(S, h, b, 0, v, fs, sh, ovf);
                     }
                 } else {
-                    const int b = s.obs_off + 5 * c;
+                    const int b = s.obs_off + 5 * c, h = hist_at<L>(S, b, 5);
                     if constexpr (sizeof(R) == 4) {
                         // |u_n| <= sqrt 2 for every n and nu (a Gaussian average
                         // of Hermite functions, Cramer's bound), so one test of
@@ -527,18 +603,18 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
                         const float4 *rc = S.ghc + 3 * (s.ghc_off + c);
                         const float W = wv * fs;
                         if (fabsf(W) < 0.5f * FX_FAST) {
-                            gh_red_stream(vlos, rc, W, S.hL, S.hM, b);
+                            gh_red_stream(vlos, rc, W, S.hL, S.hM, h);
                         } else {
                             R u[5];
                             gh_eval_rec(vlos, rc, u);
 #pragma unroll
-                            for (int m = 0; m < 5; ++m) hist_add(S, b + m, wv * u[m], fs, sh, ovf);
+                            for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
                         }
                     } else {
                         R u[5];
                         gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
 #pragma unroll
-                        for (int m = 0; m < 5; ++m) hist_add(S, b + m, wv * u[m], fs, sh, ovf);
+                        for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
                     }
                 }
             }
@@ -750,7 +826,12 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     unsigned char *p = smem;
     const int nobs = a.nobs;
     if (fl & F_SCAT) {
-        if (FX) { S.hL = (int *)p; S.hM = S.hL + nobs; S.hH = S.hM + nobs; p += 12 * ((nobs + 3) & ~3); }
+        if (FX) {
+            S.hrep = hist_copied<L> ? a.hrep : 1;
+            S.hlane = (int)threadIdx.x & (S.hrep - 1);
+            S.hL = (int *)p; S.hM = S.hL + nobs * S.hrep; S.hH = S.hM + nobs * S.hrep;
+            p += (4 + 8 * S.hrep) * ((nobs + 3) & ~3);
+        }
         else { S.h_d = (double *)p; p += 8 * ((nobs + 1) & ~1); }
     }
     if (fl & F_UPD) { S.coef = (const R *)p; p += sizeof(R) * ((nobs + 3) & ~3); }
@@ -790,7 +871,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     // so it is read after griddep_wait)
     if (fl & F_SCAT) {
         unsigned *hz = FX ? (unsigned *)S.hL : (unsigned *)S.h_d;
-        for (int k = threadIdx.x; k < (FX ? 3 : 2) * nobs; k += NT) hz[k] = 0u;
+        for (int k = threadIdx.x; k < (FX ? 1 + 2 * S.hrep : 2) * nobs; k += NT) hz[k] = 0u;
     }
     for (int k = threadIdx.x; k < a.edge_len; k += NT) {
         const R *et = (const R *)a.edge_tab;
@@ -868,17 +949,14 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     int nseg = 0;
     auto flush_hist = [&](bool last) {
         long long *sl = (long long *)a.slots + (long long)bid * nobs;
-        for (int k = threadIdx.x; k < nobs; k += NT) {
-            const long long v = (long long)(((unsigned long long)(long long)S.hH[k] << 32) +
-                                            ((unsigned long long)(long long)S.hM[k] << 16) +
-                                            (unsigned long long)(long long)S.hL[k]);
-            if (!last) { S.hL[k] = 0; S.hM[k] = 0; S.hH[k] = 0; }
-            if (a.fx_atomic) {
-                if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
-            } else {
-                sl[k] = nseg ? sl[k] + v : v;
-            }
-        }
+        if constexpr (FX)
+            fx_totals<L>(a, S, threadIdx.x >> 5, NT / 32, !last, [&](int k, long long v) {
+                if (a.fx_atomic) {
+                    if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
+                } else {
+                    sl[k] = nseg ? sl[k] + v : v;
+                }
+            });
         ++nseg;
     };
     if constexpr (PIPE) {

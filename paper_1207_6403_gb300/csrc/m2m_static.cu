@@ -250,6 +250,7 @@ int m2m_observe_static(int64_t n, const void *x, const void *y, const void *z, c
     a.fx_shift = FX_AVG_BITS + nbits - wexp;
     a.y_acc = (unsigned long long *)(base + OFF_TOT);
     a.fx_atomic = 1;
+    a.hrep = 1;
     a.err = (int *)(base + OFF_ERR);
     a.prior_kind = M2M_PRIOR_FLAT; a.nE = 1; a.nL = 1;
     const int layout = layout_of(a.sets, nsets);

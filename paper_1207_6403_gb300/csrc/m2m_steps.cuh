@@ -151,13 +151,9 @@ __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSme
             // terms per bin between flushes): this segment into the int64
             // totals
             __syncthreads();
-            for (int q = threadIdx.x; q < a.nobs; q += NT) {
-                const long long v = (long long)(((unsigned long long)(long long)S.hH[q] << 32) +
-                                                ((unsigned long long)(long long)S.hM[q] << 16) +
-                                                (unsigned long long)(long long)S.hL[q]);
-                S.hL[q] = 0; S.hM[q] = 0; S.hH[q] = 0;
+            fx_totals<L>(a, S, threadIdx.x >> 5, NT / 32, true, [&](int q, long long v) {
                 if (v) atomicAdd(a.y_acc + q, (unsigned long long)v);
-            }
+            });
             __syncthreads();
             it = 0;
         }
@@ -180,7 +176,10 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
     unsigned char *p = smem;
     const int nobs = a.nobs, nobs4 = (nobs + 3) & ~3;
     // the histogram's three parts each 16-byte aligned (vector flushes)
-    S.hL = (int *)p; S.hM = S.hL + nobs4; S.hH = S.hM + nobs4; p += 12 * nobs4;
+    S.hrep = hist_copied<L> ? a.hrep : 1;
+    S.hlane = (int)threadIdx.x & (S.hrep - 1);
+    const int nh4 = nobs4 * S.hrep;
+    S.hL = (int *)p; S.hM = S.hL + nh4; S.hH = S.hM + nh4; p += 4 * (nobs4 + 2 * nh4);
     S.coef = (const R *)p; p += 4 * nobs4;
     S.edges = (const R *)p; p += 4 * ((a.edge_len + 3) & ~3);
     S.epair = (const Pair<R> *)p; p += 8 * ((a.edge_len + 1) & ~1);
@@ -232,7 +231,7 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
                 for (int k = threadIdx.x; k < nobs; k += NT) ((R *)S.coef)[k] = __ldcg((const R *)r.coef_r + k);
             }
         }
-        for (int k = threadIdx.x; k < 3 * nobs4 / 4; k += NT) ((int4 *)S.hL)[k] = make_int4(0, 0, 0, 0);
+        for (int k = threadIdx.x; k < (nobs4 + 2 * nh4) / 4; k += NT) ((int4 *)S.hL)[k] = make_int4(0, 0, 0, 0);
         __syncthreads();
         // the GH records of this step's update
         for (int k = 0; k < a.nsets; ++k) {
@@ -292,12 +291,9 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
             // meanwhile the other warps flush the histogram into the int64
             // totals (integer atomics: any order; a warp's 32 atomics on 32
             // consecutive totals, two cache lines)
-            for (int k = (int)threadIdx.x - 32; k < nobs; k += NT - 32) {
-                const long long v = (long long)(((unsigned long long)(long long)S.hH[k] << 32) +
-                                                ((unsigned long long)(long long)S.hM[k] << 16) +
-                                                (unsigned long long)(long long)S.hL[k]);
+            fx_totals<L>(a, S, wp - 1, NT / 32 - 1, false, [&](int k, long long v) {
                 if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
-            }
+            });
         }
         round += (unsigned long long)G;
         grid_barrier(A.bar, round, A.wait_ns, a.err, !(A.test_stall && b == 0 && s == 0));
