@@ -377,8 +377,8 @@ int64_t m2m_nobs(const m2m_ctx *ctx);
 int64_t m2m_steps_taken(const m2m_ctx *ctx);
 
 /* Launch shape of the particle kernels: threads per block (FP32C: 256, 512
- * or 1024 (default; the pipelined pass needs 1024); FP64: 256 (default) or
- * 512) and blocks per SM (0 = as many as fit, at most 4).  Takes effect on
+ * or 1024 (default; the pipelined pass needs 1024); FP64: 256 or 512 (default:
+ * 512 where every SM has that many particles, else 256)) and blocks per SM (0 = as many as fit, at most 4).  Takes effect on
  * the next launch. */
 int m2m_set_launch(m2m_ctx *ctx, int32_t threads, int32_t blocks_per_sm);
 

@@ -30,6 +30,7 @@
 #include "m2m.h"
 #define M2M_COMMON_KERNELS
 #include "m2m_kernels.cuh"
+#include "m2m_pass64.cuh"
 #include "m2m_analysis.cuh"
 #include "m2m_steps.cuh"
 
@@ -57,6 +58,7 @@ struct m2m_ctx {
     int nsm;
     int smem_optin;      // shared memory a block may use on this device
     int threads, bps_req;
+    bool shape_set;      // by m2m_set_launch or the autotuner
     int nsets, nobs, npot;
     SetDev sets[MAXSETS];
     PotDev pot[MAXPOT];
@@ -127,6 +129,10 @@ struct m2m_ctx {
     long long wait_ns = 2000000000ll;      // limit of one grid-barrier wait
     int test_stall = 0;              // test only: the next launch's block 0 skips its first arrival
     long long test_wait_ns = 0;      //   and its barrier waits are limited to this
+    // FP64: what a pass leaves for the next one of the same m2m_step call
+    // ([6][n]: ln(w/w_hat), m, Gaussian factor, force), and which of it holds
+    double *d_c64 = nullptr, *d_exp = nullptr;
+    bool in_step = false, c64_lnw = false, c64_gh = false, c64_force = false;
     void *d_vm = nullptr;            // velocity moments: sums and shell edges
     size_t vm_bytes = 0;
     // particle shards (m2m_shard_*): this context holds one shard of a model
@@ -244,9 +250,15 @@ size_t pass_smem_copies(const m2m_ctx *c, int flags, int hrep) {
 // of 4.1M particles in all, 25 steps, 4.17 / 4.07 / 3.99 ms; 1M particles,
 // 25 steps, 774 / 767 / 777 us.
 int hist_copies(const m2m_ctx *c) {
-    if (c->prec != M2M_FP32C || c->threads != 1024 || c->pipe || (c->layout != 2 && c->layout != 3)) return 1;
     const size_t room = (size_t)c->smem_optin - 4096;       // the kernels' static shared memory
+    if (c->prec == M2M_FP32C && (c->threads != 1024 || c->pipe || (c->layout != 2 && c->layout != 3))) return 1;
     int r = c->launch_n >= 8ll * 1024 * c->nsm ? 32 : 8;
+    if (c->prec == M2M_FP64) {
+        // (r - 1) nobs FP64 adds when a block sums the copies: at most a
+        // fiftieth of its particles' some 180 operations
+        r = 32;
+        while (r > 1 && (double)(r - 1) * c->nobs > 3.6 * (double)c->n / c->nsm) r >>= 1;
+    }
     while (r > 1 && pass_smem_copies(c, F_STEADY | F_MINMAX, r) > room) r >>= 1;
     return r;
 }
@@ -328,6 +340,10 @@ int detect_layout(const m2m_ctx *c) {
 
 LaunchShape pick_kernel(const m2m_ctx *c) {
     int nt = c->threads;
+    // FP64, no shape asked for: 16 warps on an SM hide the FP64 latency better
+    // than 8 (2M particles 13.7 ms against 14.7 for 25 steps) where there are
+    // particles for them (20,000: 268 us against 263 for 10 steps)
+    if (c->prec == M2M_FP64 && !c->shape_set && c->n >= 512ll * c->nsm) nt = 512;
     if (c->prec == M2M_FP32C) return {pass_kernel_f32(nt, c->layout), nt};
     return {pass_kernel_f64(nt, c->layout), nt};
 }
@@ -366,6 +382,16 @@ void fill_args(const m2m_ctx *c, PassArgs &a, int flags) {
     a.sh_tab = c->sh_on ? c->d_sh_tab : nullptr; a.sh_K = c->sh_K; a.sh_row = c->sh_row;
     a.facc = (c->sh_on && !c->facc_off) ? c->d_facc : nullptr;
     a.facc_read = (flags & F_PUSH) && a.facc && c->facc_valid;
+    a.exp_tab = c->d_exp;
+    if (c->in_step && c->d_c64) {
+        a.c64_lnw = c->d_c64;
+        if (c->layout == 1 || c->layout == 2) { a.c64_m = c->d_c64 + c->n; a.c64_g = c->d_c64 + 2 * c->n; }
+        a.c64_read = (c->c64_lnw ? C64_LNW : 0) | (c->c64_gh ? C64_GH : 0);
+        if (!c->sh_on) {
+            a.facc = c->d_c64 + 3 * c->n;
+            a.facc_read = (flags & F_PUSH) && c->c64_force;
+        }
+    }
     a.cell_cache = c->d_cell_cache;
     a.cache_read = (flags & F_UPD) && c->cache_valid && c->layout != 0;
     a.cache_write = (flags & F_SCAT) && c->layout != 0;
@@ -424,8 +450,8 @@ int launch_pass(m2m_ctx *ctx, int flags, int *grid_out = nullptr) {
     if (occ < 1) return set_err(ctx, M2M_ERR_ARG, "pass needs %zu B shared memory: does not fit", sm);
     int bps = occ;
     if (ctx->bps_req > 0 && ctx->bps_req < bps) bps = ctx->bps_req;
-    long long nch = (ctx->n + (ctx->prec == M2M_FP32C ? 3 : 1)) / (ctx->prec == M2M_FP32C ? 4 : 2);
-    long long need = (nch + ks.nt - 1) / ks.nt;
+    // FP64 deals chunks of 32 particles round the blocks
+    long long need = ctx->prec == M2M_FP32C ? ((ctx->n + 3) / 4 + ks.nt - 1) / ks.nt : (ctx->n + 31) / 32;
     long long grid = (long long)ctx->nsm * bps;
     if (grid > ctx->slot_cap) grid = ctx->slot_cap;
     if (grid > need) grid = need;
@@ -441,7 +467,12 @@ int launch_pass(m2m_ctx *ctx, int flags, int *grid_out = nullptr) {
     if (flags & F_MINMAX) ctx->mm_nblocks = (int)grid;
     if (flags & F_SCAT) ctx->cache_valid = ctx->layout != 0;
     else if (flags & F_PUSH) ctx->cache_valid = false;
-    if (flags & F_PUSH) ctx->facc_valid = a.facc != nullptr;
+    if (flags & F_PUSH) ctx->facc_valid = ctx->sh_on && a.facc != nullptr;
+    if (a.c64_lnw) {
+        if (flags & (F_UPD | F_STATS)) ctx->c64_lnw = true;
+        if (flags & F_PUSH) ctx->c64_force = true;
+        if (flags & (F_SCAT | F_PUSH)) ctx->c64_gh = (flags & F_SCAT) && a.c64_m;
+    }
     if (flags & F_PUSH) ++ctx->epoch;
     if (grid_out) *grid_out = (int)grid;
     return M2M_OK;
@@ -457,8 +488,8 @@ int launch_residual(m2m_ctx *ctx, int mode, long long rec_step, int write_ring, 
     ResArgs r;
     memset(&r, 0, sizeof r);
     r.slots = ctx->d_slots; r.nblk = ctx->last_grid; r.nobs = ctx->nobs; r.y_acc = ctx->d_y_acc;
-    r.fx_atomic = ctx->fx_atomic;
     r.fixed = ctx->prec == M2M_FP32C; r.q = ctx->fx_q;
+    r.fx_atomic = r.fixed ? ctx->fx_atomic : 1;
     r.Y = ctx->d_Y; r.inv_sigma = ctx->d_isig; r.Dt = ctx->d_Dt; r.y = ctx->d_y; r.Delta = ctx->d_Delta;
     r.coef_d = ctx->d_coef_d; r.coef_r = ctx->d_coef_r; r.r_float = ctx->prec == M2M_FP32C;
     r.mode = mode; r.alpha = ctx->par.alpha; r.mu = ctx->par.mu;
@@ -467,7 +498,7 @@ int launch_residual(m2m_ctx *ctx, int mode, long long rec_step, int write_ring, 
     r.chi_slots = ctx->d_chi_slots; r.ticket = ctx->d_ticket;
     r.ring = ctx->d_ring; r.last = ctx->d_last; r.rec_step = rec_step; r.write_ring = write_ring;
     r.err = ctx->d_err;
-    const bool direct = r.fixed && r.fx_atomic;
+    const bool direct = r.fx_atomic;
     int nt = direct ? RES_NT_FX : RES_NT;
     int nb = direct ? (ctx->nobs + RES_NT_FX - 1) / RES_NT_FX : (ctx->nobs + 31) / 32;
     void *args[] = {&r};
@@ -508,6 +539,7 @@ int prior_recompute(m2m_ctx *ctx, int pass_flags) {
         k_prior_gather<<<g, 256, 0, ctx->st>>>(ctx->d_cell_ids, ctx->d_cell_mean, ctx->what, ctx->d_lnwhat, ctx->n);
         CU(cudaGetLastError());
     }
+    ctx->c64_lnw = false;           // w_hat changed
     return M2M_OK;
 }
 
@@ -638,7 +670,7 @@ void free_all(m2m_ctx *c) {
                     c->d_last, c->d_err, c->d_mm_slots, c->d_cell_ids, c->d_cell_acc, c->d_cell_cnt,
                     c->d_cell_mean, c->d_cell_cache, c->d_y_acc, c->d_sh_e2, c->d_sh_rn, c->d_sh_irn,
                     c->d_sh_tab, c->d_sh_rnd, c->d_sh_sum, c->d_facc, c->d_lnwhat, c->d_lut, c->d_pmap, c->d_psf,
-                    c->d_bar, c->d_st2, c->d_chi2, c->d_vm};
+                    c->d_bar, c->d_st2, c->d_chi2, c->d_vm, c->d_c64, c->d_exp};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -1012,7 +1044,8 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     ALLOC(ctx->d_isig, 8 * nobs);
     ALLOC(ctx->d_y, 8 * nobs); ALLOC(ctx->d_Delta, 8 * nobs); ALLOC(ctx->d_coef_d, 8 * nobs);
     ALLOC(ctx->d_coef_r, rs * nobs);
-    ALLOC(ctx->d_slots, (size_t)8 * nobs * ctx->slot_cap);
+    if (f32) ALLOC(ctx->d_slots, (size_t)8 * nobs * ctx->slot_cap);
+    if (!f32) ALLOC(ctx->d_exp, 8 * EXP_N);
     ALLOC(ctx->d_y_acc, (size_t)8 * nobs);
     ALLOC(ctx->d_stat_slots, (size_t)32 * ctx->slot_cap);
     ALLOC(ctx->d_rec_ticket, 8);
@@ -1035,6 +1068,15 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         ALLOC(ctx->d_cell_acc, 8 * (size_t)ctx->ncells);
         ALLOC(ctx->d_cell_cnt, 4 * (size_t)ctx->ncells);
         ALLOC(ctx->d_cell_mean, 8 * (size_t)ctx->ncells);
+    }
+    if (!f32) {
+        // only where it leaves the caller most of the memory; without it every
+        // pass computes these values itself
+        size_t freeb = 0, totb = 0;
+        if (cudaMemGetInfo(&freeb, &totb) == cudaSuccess && 48 * (size_t)n < freeb / 4 &&
+            cudaMalloc((void **)&ctx->d_c64, 48 * (size_t)n) != cudaSuccess)
+            ctx->d_c64 = nullptr;
+        cudaGetLastError();
     }
 #undef ALLOC
 
@@ -1086,7 +1128,10 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
                                         : cudaMemcpy(ctx->d_psf, pb.data(), pb.size(), cudaMemcpyHostToDevice);
         for (int k = 0; k < nsets; ++k)
             if (obs[k].psf_q) ctx->sets[k].psf = (const unsigned char *)ctx->d_psf + rs * psf_off[k];
-        cudaError_t es[] = {e1, e2, e3, e4, e5, e6, e7, e8, e9, e10, e11, e12};
+        double exp_h[EXP_N];
+        for (int k = 0; k < EXP_N; ++k) exp_h[k] = exp2((double)k / EXP_N);
+        cudaError_t e13 = f32 ? cudaSuccess : cudaMemcpy(ctx->d_exp, exp_h, sizeof exp_h, cudaMemcpyHostToDevice);
+        cudaError_t es[] = {e1, e2, e3, e4, e5, e6, e7, e8, e9, e10, e11, e12, e13};
         for (cudaError_t e : es)
             if (e != cudaSuccess) {
                 set_err(nullptr, M2M_ERR_CUDA, "table upload: %s", cudaGetErrorString(e));
@@ -1257,9 +1302,7 @@ int m2m_push(m2m_ctx *ctx, int64_t nsteps) {
     return M2M_OK;
 }
 
-int m2m_step(m2m_ctx *ctx, int64_t nsteps) {
-    if (!ctx || nsteps < 0) return set_err(ctx, M2M_ERR_ARG, "bad argument");
-    if (ctx->shard) return set_err(ctx, M2M_ERR_STATE, "a shard context steps through m2m_shard_*");
+static int run_steps(m2m_ctx *ctx, int64_t nsteps) {
     const bool moving = ctx->prior.kind != M2M_PRIOR_FLAT;
     for (int64_t k = 0; k < nsteps; ++k) {
         long long t1 = ctx->t + 1;
@@ -1314,6 +1357,18 @@ int m2m_step(m2m_ctx *ctx, int64_t nsteps) {
     }
     if (!ctx->lazy_update) return finish_update(ctx);
     return M2M_OK;
+}
+
+int m2m_step(m2m_ctx *ctx, int64_t nsteps) {
+    if (!ctx || nsteps < 0) return set_err(ctx, M2M_ERR_ARG, "bad argument");
+    if (ctx->shard) return set_err(ctx, M2M_ERR_STATE, "a shard context steps through m2m_shard_*");
+    // FP64 passes leave values to the next pass of this call only (the caller
+    // may change its arrays between calls)
+    ctx->c64_lnw = ctx->c64_gh = ctx->c64_force = false;
+    ctx->in_step = ctx->prec == M2M_FP64;
+    const int rc = run_steps(ctx, nsteps);
+    ctx->in_step = false;
+    return rc;
 }
 
 int m2m_set_lazy_update(m2m_ctx *ctx, int32_t on) {
@@ -1604,6 +1659,7 @@ int m2m_set_launch(m2m_ctx *ctx, int32_t threads, int32_t blocks_per_sm) {
     if (!ok || blocks_per_sm < 0 || blocks_per_sm > 4)
         return set_err(ctx, M2M_ERR_ARG, "launch shape %d threads x %d blocks/SM not supported", threads, blocks_per_sm);
     ctx->threads = threads;
+    ctx->shape_set = true;
     ctx->bps_req = blocks_per_sm;
     return M2M_OK;
 }
@@ -1644,6 +1700,7 @@ int m2m_autotune(m2m_ctx *ctx, int32_t steps_per_trial, const char *cache_path, 
                 int nt = 0, pl = 0;
                 if (pt && pp && sscanf(pt + 11, "%d", &nt) == 1 && sscanf(pp + 12, "%d", &pl) == 1 && valid(nt, pl)) {
                     ctx->threads = nt;
+                    ctx->shape_set = true;
                     ctx->bps_req = 0;
                     ctx->pipe = (pl & 1) != 0;
                     ctx->fx_atomic = (pl & 2) ? 0 : 1;
@@ -1655,6 +1712,7 @@ int m2m_autotune(m2m_ctx *ctx, int32_t steps_per_trial, const char *cache_path, 
         }
     }
     if (int rc0 = finish_update(ctx)) return rc0;
+    ctx->shape_set = true;
     const int shapes[] = {1024, 512, 256};
     const int flushes[] = {4, 2, 4 | 1, 2 | 1};
     const bool was_timing = ctx->timing;

@@ -20,6 +20,7 @@ constexpr int MAXCELLS = 16385;
 
 enum { F_UPD = 1, F_PUSH = 2, F_SCAT = 4, F_STATS = 8, F_MINMAX = 16, F_CELLS = 32 };
 enum { G_LIN = 0, G_LOG = 1, G_BIS = 2 };
+enum { C64_LNW = 1, C64_GH = 2 };
 enum { ERR_NONFINITE = 1, ERR_OVERFLOW = 2, ERR_TIMEOUT = 4 };
 
 struct SetDev {
@@ -90,6 +91,11 @@ struct PassArgs {
     double pk, pgma;                        // e_lc: a/GM, GM*a
     void *mm_slots; int mm_nblocks;         // [mm_nblocks][4] R: min E, max E, max|Lz|, pad
     const void *sh_tab; int sh_K, sh_row;   // expansion node table (R, sh_row values per node) or NULL
+    // FP64, inside one m2m_step call: what the preceding pass left for the same
+    // particles ([n] each, or null), and which of it holds (C64_* bits)
+    double *c64_lnw, *c64_m, *c64_g;        // ln(w/w_hat); m and the Gaussian factor of the GH cell
+    int c64_read;
+    const double *exp_tab;                  // FP64: 2^(j/128)
     void *facc; int facc_read;              // expansion potentials: force at the positions (R, [3][n]) or NULL
     // record of the preceding step, left by its residual to this pass (the
     // first block to finish its particles writes it; see record_warp)
@@ -301,6 +307,39 @@ __device__ __forceinline__ void fixed_add(unsigned *lo, unsigned *hi, int b, lon
 // ------------------------------------------------------------ potentials
 template <class R> struct Acc3 { R x, y, z; };
 
+// Correctly rounded double division and square root for the FP64 force, in
+// as few FP64 operations as the method allows (the pipe that bounds the pass):
+// the hardware's 20-bit reciprocal (root) approximation, one third-order
+// step, and Markstein's final correction with the exact remainder (P. W.
+// Markstein, IBM J. Res. Dev. 34 (1990) 111): q + (a - q b) y rounds to a/b
+// when q is within an ulp of it and y is 1/b to within rounding.  6 and 9
+// operations.  Operands outside 2^-500 .. 2^500 (zeros, NaN, infinities) take
+// the language's operations.
+__device__ __forceinline__ bool mid_range(double v) {
+    return (((unsigned)__double2hiint(v) >> 20) & 0x7ffu) - 523u <= 1000u;
+}
+__device__ __forceinline__ double div_rn(double a, double b) {
+    if (!(mid_range(a) && mid_range(b))) return a / b;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+    const double e = fma(-b, y, 1.0);
+    y = fma(y, fma(e, e, e), y);
+    const double q = a * y;
+    return fma(fma(-b, q, a), y, q);
+}
+__device__ __forceinline__ double sqrt_rn(double a) {
+    if (!(mid_range(a) && __double2hiint(a) >= 0)) return sqrt(a);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    double g = a * y, h = 0.5 * y;
+    const double e = fma(-g, h, 0.5), c = fma(1.5 * e, e, e);     // g = sqrt(a)(1 - e) to first order
+    g = fma(g, c, g);
+    h = fma(h, c, h);
+    return fma(fma(-g, g, a), h, g);
+}
+__device__ __forceinline__ float div_rn(float a, float b) { return a / b; }
+__device__ __forceinline__ float sqrt_rn(float a) { return sqrtf(a); }
+
 __device__ __forceinline__ float nfw_f(float r, const PotDev &p) {
     // M(r)/r^3, M = C [ln(1+u) - u/(1+u)], u = r/r_s
     float u = r * p.cf[2];
@@ -319,10 +358,10 @@ __device__ __forceinline__ double nfw_f(double r, const PotDev &p) {
     if (u < 1e-3) {
         mu = u * u * (0.5 - u * (2.0 / 3.0 - u * (0.75 - 0.8 * u)));
     } else {
-        mu = log1p(u) - u / (1.0 + u);
+        mu = log1p(u) - div_rn(u, 1.0 + u);
     }
     double r3 = r * r * r;
-    return r > 0. ? p.c[0] * mu / r3 : 0.;
+    return r > 0. ? div_rn(p.c[0] * mu, r3) : 0.;
 }
 
 // ------------------------------------------------------------ multipoles
@@ -654,9 +693,9 @@ template <class R>
 __device__ __forceinline__ void acc_hernquist(R x, R y, R z, const PotDev &p, Acc3<R> &g) {
     R GM = KC(R, p.c[0], p.cf[0]), aa = KC(R, p.c[1], p.cf[1]);
     R r2 = (x * x + y * y) + z * z;
-    R r = sqrt(r2);
+    R r = sqrt_rn(r2);
     R s = r + aa;
-    R f = r2 > R(0) ? GM / ((r * s) * s) : R(0);
+    R f = r2 > R(0) ? div_rn(GM, (r * s) * s) : R(0);
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-(f * z));
@@ -666,7 +705,7 @@ __device__ __forceinline__ void acc_log(R x, R y, R z, const PotDev &p, Acc3<R> 
     R Rc2 = KC(R, p.c[0], p.cf[0]), iq2 = KC(R, p.c[1], p.cf[1]), v0sq = KC(R, p.c[2], p.cf[2]);
     R R2 = x * x + y * y;
     R D = (Rc2 + R2) + (z * z) * iq2;
-    R f = v0sq / D;
+    R f = div_rn(v0sq, D);
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-((f * iq2) * z));
@@ -674,7 +713,7 @@ __device__ __forceinline__ void acc_log(R x, R y, R z, const PotDev &p, Acc3<R> 
 template <class R>
 __device__ __forceinline__ void acc_nfw(R x, R y, R z, const PotDev &p, Acc3<R> &g) {
     R r2 = (x * x + y * y) + z * z;
-    R f = nfw_f(sqrt(r2), p);
+    R f = nfw_f(sqrt_rn(r2), p);
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-(f * z));
@@ -687,9 +726,9 @@ template <class R>
 __device__ __forceinline__ Acc3<R> acc1_hernquist(R x, R y, R z, const PotDev &p) {
     R GM = KC(R, p.c[0], p.cf[0]), aa = KC(R, p.c[1], p.cf[1]);
     R r2 = (x * x + y * y) + z * z;
-    R r = sqrt(r2);
+    R r = sqrt_rn(r2);
     R s = r + aa;
-    R f = r2 > R(0) ? GM / ((r * s) * s) : R(0);
+    R f = r2 > R(0) ? div_rn(GM, (r * s) * s) : R(0);
     return Acc3<R>{-(f * x), -(f * y), -(f * z)};
 }
 template <class R>
@@ -697,8 +736,27 @@ __device__ __forceinline__ Acc3<R> acc1_log(R x, R y, R z, const PotDev &p) {
     R Rc2 = KC(R, p.c[0], p.cf[0]), iq2 = KC(R, p.c[1], p.cf[1]), v0sq = KC(R, p.c[2], p.cf[2]);
     R R2 = x * x + y * y;
     R D = (Rc2 + R2) + (z * z) * iq2;
-    R f = v0sq / D;
+    R f = div_rn(v0sq, D);
     return Acc3<R>{-(f * x), -(f * y), -((f * iq2) * z)};
+}
+
+// The force and the potential of an expansion component (kinds 4-6) in
+// double, for the run-time component walk: kept out of line, because inlined
+// into the walk their arithmetic was also executed where the component is
+// another one (508 FP64 instructions per particle for a push in the
+// logarithmic potential, 81 with the calls).
+static __device__ __noinline__ Acc3<double> ex_accel_call(int kind, double x, double y, double z, const PotDev &p,
+                                                   const double *sh) {
+    Acc3<double> g{0.0, 0.0, 0.0};
+    if (kind == 4) sh_accel<double>(x, y, z, sh, p, g);
+    else if (kind == 5) tri_accel<double>(x, y, z, sh, p, g);
+    else full_accel<double>(x, y, z, sh, p, g);
+    return g;
+}
+static __device__ __noinline__ double ex_phi_call(int kind, double x, double y, double z, const PotDev &p,
+                                           const double *sh) {
+    return kind == 4 ? sh_phi<double>(x, y, z, sh, p)
+         : kind == 5 ? tri_phi<double>(x, y, z, sh, p) : full_phi<double>(x, y, z, sh, p);
 }
 
 template <class R, int PK = PK_ANY>
@@ -730,6 +788,11 @@ __device__ __forceinline__ Acc3<R> accel(R x, R y, R z, const PassArgs &a, const
             acc_log<R>(x, y, z, p, g);
         } else if (p.kind == 2) {     // NFW
             acc_nfw<R>(x, y, z, p, g);
+        } else if (sizeof(R) == 8) {  // an expansion of the particles
+            const Acc3<double> e = ex_accel_call(p.kind, x, y, z, p, (const double *)sh);
+            g.x = g.x + e.x;
+            g.y = g.y + e.y;
+            g.z = g.z + e.z;
         } else if (p.kind == 4) {     // spherical harmonics of the particles
             sh_accel<R>(x, y, z, sh, p, g);
         } else if (p.kind == 5) {     // the triaxial expansion of the particles
@@ -824,6 +887,8 @@ __device__ __forceinline__ R phi_term(int kind, R x, R y, R z, const PotDev &p, 
         double u = r * p.c[2];
         double v = r > 0 ? -p.c[0] * log1p(u) / r : -p.c[0] * p.c[2];
         return (R)v;
+    } else if (sizeof(R) == 8 && kind >= 4) {
+        return (R)ex_phi_call(kind, x, y, z, p, (const double *)sh);
     } else if (kind == 4) {
         return sh_phi<R>(x, y, z, sh, p);
     } else if (kind == 5) {
@@ -950,21 +1015,6 @@ __device__ __forceinline__ void gh_eval(float vlos, const float *g, float u[5]) 
     u[3] = gs * (fmaf(2.f, E3, -3.f * m) * ISQ3);
     u[4] = gs * (fmaf(4.f, E4, fmaf(-12.f, E2, 3.f)) * ISQ24);
 }
-__device__ __forceinline__ void gh_eval(double vlos, const double *g, double u[5]) {
-    const double SQ2 = 1.4142135623730951, SQ3 = 1.7320508075688772, SQ24 = 4.898979485566356;
-    double nu = (vlos - g[0]) * g[1];
-    double c1 = g[2], t2 = g[3];
-    double gs = g[4] * exp(-0.5 * nu * nu * c1);
-    double m = nu * c1, m2 = m * m;
-    double E2 = m2 + t2;
-    double E3 = m * m2 + 3.0 * m * t2;
-    double E4 = m2 * m2 + 6.0 * m2 * t2 + 3.0 * t2 * t2;
-    u[0] = gs;
-    u[1] = gs * (SQ2 * m);
-    u[2] = gs * ((2.0 * E2 - 1.0) / SQ2);
-    u[3] = gs * ((2.0 * E3 - 3.0 * m) / SQ3);
-    u[4] = gs * ((4.0 * E4 - 12.0 * E2 + 3.0) / SQ24);
-}
 
 // The per-cell record of the compiled FP32C layouts (three float4):
 //   r[0] = (V, c1/S, -log2(e)/(2S), log2 norm), r[1] = (P0, P1, P2, P3),
@@ -1000,9 +1050,6 @@ __device__ __forceinline__ void gh_eval_rec(float vlos, const float4 *r, float u
     u[3] = g * (m * fmaf(K3, m2, c.z));
     u[4] = g * fmaf(m2, fmaf(K4, m2, c.w), (c.w * c.w) * C4);
 }
-
-__device__ __forceinline__ float gh_exp(float x) { return exp_ftz(x); }
-__device__ __forceinline__ double gh_exp(double x) { return exp(x); }
 
 // Philox4x32 with 10 rounds (Salmon, Moraes, Dror and Shaw, SC'11): the
 // round multipliers and Weyl key increments of that publication.

@@ -292,20 +292,20 @@ __device__ __forceinline__ void stage(T *dst, const T *src, int n, int tid, int 
 }
 
 // ----------------------------------------------------------------- k_pass
-// Dynamic shared memory of pass_body (host side; the same order and
-// rounding as the carve-up at the top of pass_body, without the pipeline's
+// Dynamic shared memory of pass_body and, FP64, of pass64_body (host side;
+// the same order and rounding as the carve-up at their top, without the pipeline's
 // stage buffers).  sh_len: SH node-table values staged when the pass pushes.
 inline size_t pass_smem_bytes(bool f32, int layout, int flags, int nobs, int edge_len, int gh_len, int sh_len,
                               int nE, int nL, int ncells, int pmap_len = 0, int hrep = 1) {
     const size_t rs = f32 ? 4 : 8;
     size_t b = 0;
-    if (flags & F_SCAT) b += f32 ? (4 + 8 * (size_t)hrep) * ((nobs + 3) & ~3) : 8 * (size_t)((nobs + 1) & ~1);
-    if (flags & F_UPD) b += rs * (size_t)((nobs + 3) & ~3);
-    b += rs * (size_t)((edge_len + 3) & ~3);
-    b += 2 * rs * (size_t)((edge_len + 1) & ~1);                     // edge pairs
+    if (flags & F_SCAT) b += f32 ? (4 + 8 * (size_t)hrep) * ((nobs + 3) & ~3) : 8 * (size_t)hrep * ((nobs + 1) & ~1);
+    if ((f32 || layout == 0) && (flags & F_UPD)) b += rs * (size_t)((nobs + 3) & ~3);
+    if (f32 || layout == 0) b += rs * (size_t)((edge_len + 3) & ~3);
+    if (f32 || layout != 0) b += 2 * rs * (size_t)((edge_len + 1) & ~1);   // edge pairs (FP64: their keys)
     b += rs * (size_t)((gh_len + 3) & ~3);
     if (f32 && layout != 0) b += 48 * (size_t)(gh_len / 5);          // combined GH records
-    else if (flags & F_UPD) b += rs * (size_t)((gh_len + 3) & ~3);
+    else if (!f32 && layout != 0 && (flags & F_UPD)) b += rs * (size_t)((gh_len + 3) & ~3);
     if (f32 && layout == 1) b += 2 * (size_t)((pmap_len + 7) & ~7);   // pixel -> aperture table
     if (sh_len && (flags & (F_PUSH | F_MINMAX | F_CELLS))) b += rs * (size_t)((sh_len + 3) & ~3);
     if (flags & F_CELLS) {
@@ -331,10 +331,8 @@ template <class R>
 struct PassSmem {
     int *hL, *hM, *hH;       // FP32C histogram: V = H * 2^32 + M * 2^16 + L per bin (exact fixed point)
     int hrep, hlane;         //   copies of L and M, and this lane's copy (see hist_copies)
-    double *h_d;             // FP64 histogram
     const R *coef, *edges, *gh;
     const Pair<R> *epair;    // (e[k], e[k+1]) for every edge-table index k
-    const R *gpoly;          // per GH cell: norm * sum_n coef_n E[H_n] as a quartic in m
     const float4 *ghc;       // FP32C compiled layouts: per GH cell the three float4 of gh_record
     R *pe, *pl;
     float *gp;
@@ -405,7 +403,7 @@ __device__ __forceinline__ R obs_dot(const PassArgs &a, const PassSmem<R> &S, R 
             int c;
             if (cached) {
                 c = (int)((cc >> s.cshift) & (unsigned)s.cmask) - 1;
-            } else if (sizeof(R) == 4 && L == 1 && k == 1 && s.pmap_len) {
+            } else if (L == 1 && k == 1 && s.pmap_len) {
                 c = c0 >= 0 ? (int)S.pmap[c0] : -1;                       // aligned with set 0's pixels
             } else {
                 R Xk = X, Yk = Ys;
@@ -421,30 +419,17 @@ __device__ __forceinline__ R obs_dot(const PassArgs &a, const PassSmem<R> &S, R 
                 } else {
                     // sum_n coef_n u_n(nu) = exp(-nu m / 2) * P(m), m = nu c1,
                     // with the quartic P of this cell built in the prologue
-                    if constexpr (sizeof(R) == 4) {
-                        // the record of gh_record: the norm in the exponent
-                        const float4 *r = S.ghc + 3 * (s.ghc_off + c);
-                        const float4 g0 = r[0], g1 = r[1];
-                        const float P4 = r[2].x;
-                        const float dv = vlos - g0.x, m = dv * g0.y;
-                        const float e = ex2_ftz(fmaf(dv * m, g0.z, g0.w));
-                        float q = fmaf(P4, m, g1.w);
-                        q = fmaf(q, m, g1.z);
-                        q = fmaf(q, m, g1.y);
-                        q = fmaf(q, m, g1.x);
-                        dot = dot + e * q;
-                    } else {
-                        const R *g = S.gh + s.gh_off + 5 * c;
-                        const R *P = S.gpoly + s.gh_off + 5 * c;
-                        const R nu = (vlos - g[0]) * g[1];
-                        const R m = nu * g[2];
-                        const R e = gh_exp(R(-0.5) * nu * m);
-                        R q = fma(P[4], m, P[3]);
-                        q = fma(q, m, P[2]);
-                        q = fma(q, m, P[1]);
-                        q = fma(q, m, P[0]);
-                        dot = dot + e * q;
-                    }
+                    // (the record of gh_record: the norm in the exponent)
+                    const float4 *r = S.ghc + 3 * (s.ghc_off + c);
+                    const float4 g0 = r[0], g1 = r[1];
+                    const float P4 = r[2].x;
+                    const float dv = vlos - g0.x, m = dv * g0.y;
+                    const float e = ex2_ftz(fmaf(dv * m, g0.z, g0.w));
+                    float q = fmaf(P4, m, g1.w);
+                    q = fmaf(q, m, g1.z);
+                    q = fmaf(q, m, g1.y);
+                    q = fmaf(q, m, g1.x);
+                    dot = dot + e * q;
                 }
             }
         });
@@ -467,8 +452,7 @@ __device__ __forceinline__ void gh_quartic(R t2, R nrm, R cf0, R cf1, R cf2, R c
 }
 
 struct ThreadAcc {
-    double s_d, w_d;     // FP64 path
-    float s_f, w_f;      // FP32C path
+    float s_f, w_f;
     bool ovf, bad;
 };
 
@@ -485,13 +469,6 @@ __device__ __forceinline__ void hist_add(const PassSmem<float> &S, int i, int b,
                                          ThreadAcc &t) {
     fx_red(S.hL, S.hM, S.hH, i + m, b + m, v, fs, sh, t.ovf);
 }
-__device__ __forceinline__ void hist_add(const PassSmem<double> &S, int, int b, int m, double v, float, int,
-                                         ThreadAcc &) {
-    atomicAdd(S.h_d + b + m, v);
-}
-template <int L>
-__device__ __forceinline__ int hist_at(const PassSmem<double> &, int b, int) { return b; }
-
 // The exact totals H * 2^32 + M * 2^16 + L of the block's FP32C histogram,
 // f(j, total) for every observable j, by `nw` warps of which this is `w`
 // (whole warps, after a barrier); clear: the histogram is zeroed for the next
@@ -575,7 +552,7 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
             R Xk = X, Yk = Ys;
             if (L == 4 && s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);       // seeing: lookup-table layout
             int c;
-            if (sizeof(R) == 4 && L == 1 && k == 1 && s.pmap_len)          // aligned with set 0's pixels
+            if (L == 1 && k == 1 && s.pmap_len)          // aligned with set 0's pixels
                 c = c0 >= 0 ? (int)S.pmap[c0] : -1;
             else
                 c = cell_t<R, g>(s, S.epair, x, y, z, Xk, Yk);
@@ -585,34 +562,23 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
                 if constexpr (q == M2M_Q_MASS || q == M2M_Q_VLOS2) {
                     const R v = q == M2M_Q_MASS ? wv : wv * (vlos * vlos);
                     const int b = s.obs_off + c, h = hist_at<L>(S, b, 1);
-                    if constexpr (sizeof(R) == 4) {
-                        const float Sv = v * fs;
-                        if (fabsf(Sv) < FX_FAST) fx_red_fast(S.hL, S.hM, h, Sv);
-                        else hist_add(S, h, b, 0, v, fs, sh, ovf);
-                    } else {
-                        hist_add(S, h, b, 0, v, fs, sh, ovf);
-                    }
+                    const float Sv = v * fs;
+                    if (fabsf(Sv) < FX_FAST) fx_red_fast(S.hL, S.hM, h, Sv);
+                    else hist_add(S, h, b, 0, v, fs, sh, ovf);
                 } else {
                     const int b = s.obs_off + 5 * c, h = hist_at<L>(S, b, 5);
-                    if constexpr (sizeof(R) == 4) {
-                        // |u_n| <= sqrt 2 for every n and nu (a Gaussian average
-                        // of Hermite functions, Cramer's bound), so one test of
-                        // the weight decides the fast path for all five terms,
-                        // each added as soon as it is formed: (w 2^sh) u_n =
-                        // (w u_n) 2^sh exactly
-                        const float4 *rc = S.ghc + 3 * (s.ghc_off + c);
-                        const float W = wv * fs;
-                        if (fabsf(W) < 0.5f * FX_FAST) {
-                            gh_red_stream(vlos, rc, W, S.hL, S.hM, h);
-                        } else {
-                            R u[5];
-                            gh_eval_rec(vlos, rc, u);
-#pragma unroll
-                            for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
-                        }
+                    // |u_n| <= sqrt 2 for every n and nu (a Gaussian average
+                    // of Hermite functions, Cramer's bound), so one test of
+                    // the weight decides the fast path for all five terms,
+                    // each added as soon as it is formed: (w 2^sh) u_n =
+                    // (w u_n) 2^sh exactly
+                    const float4 *rc = S.ghc + 3 * (s.ghc_off + c);
+                    const float W = wv * fs;
+                    if (fabsf(W) < 0.5f * FX_FAST) {
+                        gh_red_stream(vlos, rc, W, S.hL, S.hM, h);
                     } else {
                         R u[5];
-                        gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
+                        gh_eval_rec(vlos, rc, u);
 #pragma unroll
                         for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
                     }
@@ -651,28 +617,13 @@ __device__ __forceinline__ double upd_weight(double w, float lnwh, float dot, co
     L1 = L + d;
     return wn;
 }
-__device__ __forceinline__ double upd_weight(double w, double what, double dot, const PassArgs &a, double &wnd, double &L1) {
-    double L = log(w / what);
-    double G = a.mu * (-L - a.ent_c) - dot;
-    double d = a.eps_dt * G;
-    double wn = w * exp(d);
-    wnd = wn;
-    L1 = L + d;
-    return wn;
-}
-
 __device__ __forceinline__ void acc_stats(ThreadAcc &t, float wnf, float L1) {
     t.s_f = fmaf(-wnf, L1, t.s_f);
     t.w_f += wnf;
 }
-__device__ __forceinline__ void acc_stats(ThreadAcc &t, double wnd, double L1) {
-    t.s_d += -wnd * L1;
-    t.w_d += wnd;
-}
 __device__ __forceinline__ float to_r(double v, float *) { return d2f_fast(v); }
 __device__ __forceinline__ double to_r(double v, double *) { return v; }
 __device__ __forceinline__ float rlog_ratio(double w, float lnwh, float *) { return __logf(d2f_fast(w)) - lnwh; }
-__device__ __forceinline__ double rlog_ratio(double w, double what, double *) { return log(w / what); }
 
 template <class R>
 __device__ __forceinline__ void cell_add(const PassArgs &a, const PassSmem<R> &S, int c, double wv, bool &ovf);
@@ -693,17 +644,17 @@ __device__ __forceinline__ void cell_add<double>(const PassArgs &a, const PassSm
 template <class R, int L, int FL, int PK>
 __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S, int i,
                                          R &x, R &y, R &z, R &vx, R &vy, R &vz, double &w, R what,
-                                         unsigned cc, ThreadAcc &t, R &emin, R &emax, R &lzm, float fs,
+                                         unsigned cc, ThreadAcc &t, float fs,
                                          long long epoch, bool cache_read) {
-    // what: FP32C ln w_hat, FP64 w_hat; epoch: pushes the positions have had
+    // what: ln w_hat; epoch: pushes the positions have had
     // at the start of this pass; cache_read: cc holds the cells at x
     const int fl = FL ? FL : a.flags;
     const R sn = KC(R, a.sin_i, a.f_sin_i), cs = KC(R, a.cos_i, a.f_cos_i);
     double wn = w;
-    // FP32C, a weight in the normal float range: the float arithmetic of
+    // a weight in the normal float range: the float arithmetic of
     // the update and the entropy on the two words of the double directly
     bool fast = false;
-    if constexpr (sizeof(R) == 4) {
+    {
         const unsigned hi = (unsigned)__double2hiint(w), lo = (unsigned)__double2loint(w);
         fast = w_normal(hi);
         if (fast && (fl & (F_UPD | F_STATS))) {
@@ -750,15 +701,11 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
         // the scattered weight is a function of the stored (double) weight
         // alone, whichever pass applied the update
         R wv;
-        if constexpr (sizeof(R) == 4) {
-            // the truncated float in the normal range; 0 below it (d2f_fast
-            // gives 0 there too); beyond it no term is representable
-            const unsigned hn = (unsigned)__double2hiint(wn);
-            wv = w_normal(hn) ? w_to_float(hn, (unsigned)__double2loint(wn)) : 0.f;
-            if (hn - 0x47F00000u < 0x38000000u) t.ovf = true;   // 2^128 <= wn < inf
-        } else {
-            wv = to_r(wn, (R *)nullptr);
-        }
+        // the truncated float in the normal range; 0 below it (d2f_fast
+        // gives 0 there too); beyond it no term is representable
+        const unsigned hn = (unsigned)__double2hiint(wn);
+        wv = w_normal(hn) ? w_to_float(hn, (unsigned)__double2loint(wn)) : 0.f;
+        if (hn - 0x47F00000u < 0x38000000u) t.ovf = true;   // 2^128 <= wn < inf
         // the scatter sees the positions after this pass's push, if any
         const unsigned packed = scatter<R, L>(a, S, x, y, z, X, Ys, vlos, wv, fs, t, i,
                                               epoch + ((fl & F_PUSH) ? 1 : 0));
@@ -769,26 +716,20 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
     if (fl & F_MINMAX) {
         R E, Lz;
         energy_lz<R, PK>(x, y, z, vx, vy, vz, a, S.sh, E, Lz);
-        if constexpr (sizeof(R) == 4) {
-            // FP32C: the warp's min E, max E, max |L_z| as order-preserving
-            // integer keys (one warp reduction each), then the block's by
-            // shared-memory atomics: nothing carried across the particle loop
-            const bool ok = E == E;
-            const int kE = ok ? fkey((float)E) : 0;
-            const float al = fabsf((float)Lz);
-            const unsigned m = __activemask();
-            const int r0 = __reduce_min_sync(m, ok ? kE : INT_MAX);
-            const int r1 = __reduce_max_sync(m, ok ? kE : INT_MIN);
-            const int r2 = __reduce_max_sync(m, al == al ? __float_as_int(al) : 0);
-            if ((int)(threadIdx.x & 31) == __ffs(m) - 1) {
-                atomicMin(S.mmk, r0);
-                atomicMax(S.mmk + 1, r1);
-                atomicMax(S.mmk + 2, r2);
-            }
-        } else {
-            emin = fmin(emin, E);
-            emax = fmax(emax, E);
-            lzm = fmax(lzm, fabs(Lz));
+        // FP32C: the warp's min E, max E, max |L_z| as order-preserving
+        // integer keys (one warp reduction each), then the block's by
+        // shared-memory atomics: nothing carried across the particle loop
+        const bool ok = E == E;
+        const int kE = ok ? fkey((float)E) : 0;
+        const float al = fabsf((float)Lz);
+        const unsigned m = __activemask();
+        const int r0 = __reduce_min_sync(m, ok ? kE : INT_MAX);
+        const int r1 = __reduce_max_sync(m, ok ? kE : INT_MIN);
+        const int r2 = __reduce_max_sync(m, al == al ? __float_as_int(al) : 0);
+        if ((int)(threadIdx.x & 31) == __ffs(m) - 1) {
+            atomicMin(S.mmk, r0);
+            atomicMax(S.mmk + 1, r1);
+            atomicMax(S.mmk + 2, r2);
         }
     }
     if (fl & F_CELLS) {
@@ -818,43 +759,33 @@ constexpr int FX_AVG_BITS = 25;
 template <class R, int NT, int L, int PIPE, int FL = 0, int PK = PK_ANY>
 __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, const int nblk) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double red[32];
     __shared__ __align__(8) unsigned long long bars[PIPE ? 2 * PIPE_STAGES : 1];   // full[], empty[]
-    constexpr bool FX = sizeof(R) == 4;
+    static_assert(sizeof(R) == 4, "the FP64 pass is pass64_body");
     const int fl = FL ? FL : a.flags;
     PassSmem<R> S{};
     unsigned char *p = smem;
     const int nobs = a.nobs;
     if (fl & F_SCAT) {
-        if (FX) {
-            S.hrep = hist_copied<L> ? a.hrep : 1;
-            S.hlane = (int)threadIdx.x & (S.hrep - 1);
-            S.hL = (int *)p; S.hM = S.hL + nobs * S.hrep; S.hH = S.hM + nobs * S.hrep;
-            p += (4 + 8 * S.hrep) * ((nobs + 3) & ~3);
-        }
-        else { S.h_d = (double *)p; p += 8 * ((nobs + 1) & ~1); }
+        S.hrep = hist_copied<L> ? a.hrep : 1;
+        S.hlane = (int)threadIdx.x & (S.hrep - 1);
+        S.hL = (int *)p; S.hM = S.hL + nobs * S.hrep; S.hH = S.hM + nobs * S.hrep;
+        p += (4 + 8 * S.hrep) * ((nobs + 3) & ~3);
     }
     if (fl & F_UPD) { S.coef = (const R *)p; p += sizeof(R) * ((nobs + 3) & ~3); }
     S.edges = (const R *)p; p += sizeof(R) * ((a.edge_len + 3) & ~3);
     S.epair = (const Pair<R> *)p; p += 2 * sizeof(R) * ((a.edge_len + 1) & ~1);
     S.gh = (const R *)p; p += sizeof(R) * ((a.gh_len + 3) & ~3);
-    constexpr bool GHC = FX && L != 0;      // combined GH records instead of gh + gpoly
+    constexpr bool GHC = L != 0;      // combined GH records instead of gh + gpoly
     if (GHC) { S.ghc = (const float4 *)p; p += 48 * (a.gh_len / 5); }
-    else if (fl & F_UPD) { S.gpoly = (const R *)p; p += sizeof(R) * ((a.gh_len + 3) & ~3); }
-    if (FX && L == 1) { S.pmap = (const short *)p; p += 2 * ((a.sets[1].pmap_len + 7) & ~7); }
+    if (L == 1) { S.pmap = (const short *)p; p += 2 * ((a.sets[1].pmap_len + 7) & ~7); }
     const int sh_len = (a.sh_tab && (fl & (F_PUSH | F_MINMAX | F_CELLS))) ? a.sh_row * a.sh_K : 0;
     if (sh_len) { S.sh = (const R *)p; p += sizeof(R) * ((sh_len + 3) & ~3); }
     if (fl & F_CELLS) {
         S.pe = (R *)p; p += sizeof(R) * ((a.nE + 4) & ~3);
         S.pl = (R *)p; p += sizeof(R) * ((a.nL + 4) & ~3);
         S.gp = (float *)p; p += 16;
-        if (FX) {
-            S.c_lo = (unsigned *)p; S.c_hi = S.c_lo + a.ncells; S.c_cnt = S.c_hi + a.ncells;
-            p += 12 * ((a.ncells + 3) & ~3);
-        } else {
-            S.c_d = (double *)p; p += 8 * ((a.ncells + 1) & ~1);
-            S.c_lo = (unsigned *)p; p += 4 * ((a.ncells + 3) & ~3);   // counts
-        }
+        S.c_lo = (unsigned *)p; S.c_hi = S.c_lo + a.ncells; S.c_cnt = S.c_hi + a.ncells;
+        p += 12 * ((a.ncells + 3) & ~3);
     }
     unsigned char *stages = p;        // PIPE: PIPE_STAGES chunk buffers of NT particles
     if constexpr (PIPE) {
@@ -870,8 +801,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     // are fixed at m2m_init; everything else a preceding kernel may write,
     // so it is read after griddep_wait)
     if (fl & F_SCAT) {
-        unsigned *hz = FX ? (unsigned *)S.hL : (unsigned *)S.h_d;
-        for (int k = threadIdx.x; k < (FX ? 1 + 2 * S.hrep : 2) * nobs; k += NT) hz[k] = 0u;
+        for (int k = threadIdx.x; k < (1 + 2 * S.hrep) * nobs; k += NT) S.hL[k] = 0;
     }
     for (int k = threadIdx.x; k < a.edge_len; k += NT) {
         const R *et = (const R *)a.edge_tab;
@@ -883,11 +813,11 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
         ((Pair<R> *)S.epair)[k] = pr;
     }
     stage<2>((R *)S.gh, (const R *)a.gh_tab, a.gh_len, threadIdx.x, NT);
-    if (FX && L == 1) stage<1>((short *)S.pmap, a.sets[1].pmap, a.sets[1].pmap_len, threadIdx.x, NT);
+    if (L == 1) stage<1>((short *)S.pmap, a.sets[1].pmap, a.sets[1].pmap_len, threadIdx.x, NT);
     griddep_wait();
     if (fl & F_UPD) stage<4>((R *)S.coef, (const R *)a.coef, nobs, threadIdx.x, NT);
     if (sh_len) stage<4>((R *)S.sh, (const R *)a.sh_tab, sh_len, threadIdx.x, NT);
-    if (L != 0 && (GHC || (fl & F_UPD))) {
+    if constexpr (GHC) {
         // E[H_n] over N(m, t2) as polynomials in m (van der Marel & Franx
         // H_0..H_4), weighted by this step's coefficients of the cell (0
         // in a pass without an update; FP32C keeps them with the cell's GH
@@ -901,18 +831,13 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
                 R P[5] = {R(0), R(0), R(0), R(0), R(0)};
                 if (fl & F_UPD) {
                     const R *cf = (const R *)a.coef + st.obs_off + 5 * c;
-                    // the compiled FP32C record carries the norm in its exponent
-                    gh_quartic<R>(t2, GHC ? R(1) : nrm, cf[0], cf[1], cf[2], cf[3], cf[4], P);
+                    // the record carries the norm in its exponent
+                    gh_quartic<R>(t2, R(1), cf[0], cf[1], cf[2], cf[3], cf[4], P);
                 }
-                if constexpr (GHC) {
-                    float4 rec[3];
-                    gh_record(g[0], g[1], g[2], t2, nrm, (const float *)P, rec);
-                    float4 *rc = (float4 *)S.ghc + 3 * (st.ghc_off + c);
-                    rc[0] = rec[0]; rc[1] = rec[1]; rc[2] = rec[2];
-                } else {
-                    R *Pd = (R *)S.gpoly + st.gh_off + 5 * c;
-                    for (int q = 0; q < 5; ++q) Pd[q] = P[q];
-                }
+                float4 rec[3];
+                gh_record(g[0], g[1], g[2], t2, nrm, (const float *)P, rec);
+                float4 *rc = (float4 *)S.ghc + 3 * (st.ghc_off + c);
+                rc[0] = rec[0]; rc[1] = rec[1]; rc[2] = rec[2];
             }
         }
     }
@@ -922,25 +847,19 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
         mmk[0] = fkey(INFINITY); mmk[1] = fkey(-INFINITY); mmk[2] = 0;
     }
     if (fl & F_CELLS) {
-        if (FX) {
-            for (int k = threadIdx.x; k < 3 * a.ncells; k += NT) S.c_lo[k] = 0u;   // lo, hi, cnt
-        } else {
-            for (int k = threadIdx.x; k < a.ncells; k += NT) { S.c_d[k] = 0.0; S.c_lo[k] = 0u; }
-        }
+        for (int k = threadIdx.x; k < 3 * a.ncells; k += NT) S.c_lo[k] = 0u;   // lo, hi, cnt
         prior_setup<R>(a, S.pe, S.pl, S.gp);
     }
     __syncthreads();
 
-    ThreadAcc t{0.0, 0.0, 0.f, 0.f, false, false};
-    R emin = R(INFINITY), emax = R(-INFINITY), lzm = R(0);
+    ThreadAcc t{0.f, 0.f, false, false};
     const float fs = a.fx_shift <= 127 ? __int_as_float((a.fx_shift + 127) << 23) : INFINITY;
     const long long n = a.n;
     R *px = (R *)a.x, *py = (R *)a.y, *pz = (R *)a.z, *pvx = (R *)a.vx, *pvy = (R *)a.vy, *pvz = (R *)a.vz;
     const bool wr_pos = (fl & F_PUSH) != 0;
     const bool wr_w = (fl & F_UPD) != 0;
     const bool need_what = (fl & (F_UPD | F_STATS)) != 0;
-    // FP32C reads ln w_hat (float, kept by the library), FP64 w_hat
-    const R *pwh = FX ? (const R *)a.lnwhat : (const R *)a.what;
+    const R *pwh = (const R *)a.lnwhat;
     const bool need_cc = L != 0 && a.cache_read && (fl & F_UPD);
     // FP32C histogram flush (all threads, after a barrier): the exact totals
     // H * 2^32 + M * 2^16 + L of this segment go into the global totals with
@@ -949,14 +868,13 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     int nseg = 0;
     auto flush_hist = [&](bool last) {
         long long *sl = (long long *)a.slots + (long long)bid * nobs;
-        if constexpr (FX)
-            fx_totals<L>(a, S, threadIdx.x >> 5, NT / 32, !last, [&](int k, long long v) {
-                if (a.fx_atomic) {
-                    if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
-                } else {
-                    sl[k] = nseg ? sl[k] + v : v;
-                }
-            });
+        fx_totals<L>(a, S, threadIdx.x >> 5, NT / 32, !last, [&](int k, long long v) {
+            if (a.fx_atomic) {
+                if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
+            } else {
+                sl[k] = nseg ? sl[k] + v : v;
+            }
+        });
         ++nseg;
     };
     if constexpr (PIPE) {
@@ -1037,7 +955,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
                 if (need_cc) cc = a.cell_cache[i];
             }
             if (i < (int)n) {
-                particle<R, L, FL, PK>(a, S, i, x, y, z, vx, vy, vz, w, wh, cc, t, emin, emax, lzm, fs, a.epoch,
+                particle<R, L, FL, PK>(a, S, i, x, y, z, vx, vy, vz, w, wh, cc, t, fs, a.epoch,
                                        a.cache_read != 0);
                 if (wr_pos) {
                     __stcs(px + i, x); __stcs(py + i, y); __stcs(pz + i, z);
@@ -1045,7 +963,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
                 }
                 if (wr_w) __stcs(a.w + i, w);
             }
-            if (FX && (fl & F_SCAT) && ++it == FX_SEG / NT && c + nblk < nch) {
+            if ((fl & F_SCAT) && ++it == FX_SEG / NT && c + nblk < nch) {
                 __syncthreads();
                 flush_hist(false);
                 __syncthreads();
@@ -1096,7 +1014,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
                 if (need_cc) ncc = a.cell_cache[j];
             }
             if (i < (int)n) {
-                particle<R, L, FL, PK>(a, S, i, x, y, z, vx, vy, vz, w, wh, cc, t, emin, emax, lzm, fs, a.epoch,
+                particle<R, L, FL, PK>(a, S, i, x, y, z, vx, vy, vz, w, wh, cc, t, fs, a.epoch,
                                        a.cache_read != 0);
                 if (wr_pos) {
                     __stcs(px + i, x); __stcs(py + i, y); __stcs(pz + i, z);
@@ -1105,7 +1023,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
                 if (wr_w) __stcs(a.w + i, w);
             }
             x = nx; y = ny; z = nz; vx = nvx; vy = nvy; vz = nvz; w = nw; wh = nwh; cc = ncc;
-            if (FX && (fl & F_SCAT) && ++it == FX_SEG / NT && base + stride < (int)n) {
+            if ((fl & F_SCAT) && ++it == FX_SEG / NT && base + stride < (int)n) {
                 __syncthreads();
                 flush_hist(false);
                 __syncthreads();
@@ -1125,72 +1043,31 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     griddep_launch();
     __syncthreads();
     // epilogue: flush the block-private histograms and partial sums
-    if (fl & F_SCAT) {
-        if (FX) {
-            flush_hist(true);
-        } else {
-            double *sl = (double *)a.slots + (long long)bid * nobs;
-            for (int k = threadIdx.x; k < nobs; k += NT) sl[k] = S.h_d[k];
-        }
-    }
+    if (fl & F_SCAT) flush_hist(true);
     if (fl & F_CELLS) {
-        if (FX) {
-            for (int k = threadIdx.x; k < a.ncells; k += NT) {
-                unsigned cn = S.c_cnt[k];
-                if (cn) {
-                    long long v = (long long)(((unsigned long long)S.c_hi[k] << 32) | (unsigned long long)S.c_lo[k]);
-                    atomicAdd((unsigned long long *)a.cell_acc + k, (unsigned long long)v);
-                    atomicAdd(a.cell_cnt + k, cn);
-                }
-            }
-        } else {
-            for (int k = threadIdx.x; k < a.ncells; k += NT) {
-                unsigned cn = S.c_lo[k];
-                if (cn) {
-                    atomicAdd((double *)a.cell_acc + k, S.c_d[k]);
-                    atomicAdd(a.cell_cnt + k, cn);
-                }
+        for (int k = threadIdx.x; k < a.ncells; k += NT) {
+            unsigned cn = S.c_cnt[k];
+            if (cn) {
+                long long v = (long long)(((unsigned long long)S.c_hi[k] << 32) | (unsigned long long)S.c_lo[k]);
+                atomicAdd((unsigned long long *)a.cell_acc + k, (unsigned long long)v);
+                atomicAdd(a.cell_cnt + k, cn);
             }
         }
     }
     if (fl & F_STATS) {
         double s_tot = 0.0, w_tot = 0.0;
-        if (FX) {
-            __shared__ float red2[128];
-            block_sum2_ff(t.s_f, t.w_f, red2, s_tot, w_tot);
-        } else {
-            s_tot = block_sum(t.s_d, red);
-            w_tot = block_sum(t.w_d, red);
-        }
+        __shared__ float red2[128];
+        block_sum2_ff(t.s_f, t.w_f, red2, s_tot, w_tot);
         if (threadIdx.x == 0) {
             a.stat_slots[2 * bid] = s_tot;
             a.stat_slots[2 * bid + 1] = w_tot;
         }
     }
-    if ((fl & F_MINMAX) && FX) {
+    if (fl & F_MINMAX) {
         __syncthreads();
         if (threadIdx.x == 0) {
             R *o = (R *)a.mm_slots + 4 * bid;
             o[0] = fkey_inv(S.mmk[0]); o[1] = fkey_inv(S.mmk[1]); o[2] = __int_as_float(S.mmk[2]); o[3] = R(0);
-        }
-    } else if (fl & F_MINMAX) {
-        __shared__ R mm[3][32];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            emin = fmin(emin, __shfl_xor_sync(0xffffffffu, emin, o));
-            emax = fmax(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-            lzm = fmax(lzm, __shfl_xor_sync(0xffffffffu, lzm, o));
-        }
-        int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-        if (lane == 0) { mm[0][wp] = emin; mm[1][wp] = emax; mm[2][wp] = lzm; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            R e0 = mm[0][0], e1 = mm[1][0], l2 = mm[2][0];
-            for (int k = 1; k < NT / 32; ++k) {
-                e0 = fmin(e0, mm[0][k]); e1 = fmax(e1, mm[1][k]); l2 = fmax(l2, mm[2][k]);
-            }
-            R *o = (R *)a.mm_slots + 4 * bid;
-            o[0] = e0; o[1] = e1; o[2] = l2; o[3] = R(0);
         }
     }
     if (t.ovf) atomicOr(a.err, ERR_OVERFLOW);
@@ -1275,9 +1152,10 @@ __device__ __forceinline__ double block_sum_strided(const double *v, int stride,
     return block_sum(s, red);
 }
 
-// FP32C (fx_atomic): one thread per observable in small blocks; the totals
-// are exact integers already summed by the pass's atomics (re-zeroed here
-// for the next scatter).  Slots (FP64, or FP32C without atomics): 32
+// Totals (fx_atomic): one thread per observable in small blocks; the totals
+// are already summed by the pass's atomics, exact integers in FP32C and
+// doubles in FP64 (re-zeroed here for the next scatter; reducing FP64 slots
+// of every block instead took 31 us for 6096 observables, this 5).  Slots (FP32C without atomics): 32
 // observables per block (lane = observable), the warps split the per-block
 // slots with four independent accumulators each, in a fixed order.  The
 // per-observable arithmetic is FP64 (slow on this part), so it is spread
@@ -1291,12 +1169,11 @@ __device__ __forceinline__ void residual_body(const ResArgs &a, const int bid, c
     griddep_launch();          // the next pass may stage its fixed tables meanwhile
     constexpr int NW = RES_NT / 32;
     __shared__ unsigned long long si[NW][32];
-    __shared__ double sd[NW][32];
     __shared__ double wred[3][NW];
     __shared__ int s_last;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
-    const bool direct = a.fixed && a.fx_atomic;
+    const bool direct = a.fx_atomic;
     const int j = direct ? bid * blockDim.x + threadIdx.x : bid * 32 + lane;
     bool have = false;
     double yv = 0.0;
@@ -1304,42 +1181,26 @@ __device__ __forceinline__ void residual_body(const ResArgs &a, const int bid, c
         if (j < a.nobs) {
             const unsigned long long tot = a.y_acc[j];
             a.y_acc[j] = 0ull;
-            yv = (double)(long long)tot * a.q;
+            yv = a.fixed ? (double)(long long)tot * a.q : __longlong_as_double((long long)tot);
             have = true;
         }
     } else {
         if (j < a.nobs) {
-            if (a.fixed) {
-                const long long *sl = (const long long *)a.slots + j;
-                unsigned long long acc[4] = {0, 0, 0, 0};
-                int b = wp;
-                for (; b + 3 * nw < a.nblk; b += 4 * nw) {
+            const long long *sl = (const long long *)a.slots + j;
+            unsigned long long acc[4] = {0, 0, 0, 0};
+            int b = wp;
+            for (; b + 3 * nw < a.nblk; b += 4 * nw) {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) acc[u] += (unsigned long long)sl[(long long)(b + u * nw) * a.nobs];
-                }
-                for (; b < a.nblk; b += nw) acc[0] += (unsigned long long)sl[(long long)b * a.nobs];
-                si[wp][lane] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            } else {
-                const double *sl = (const double *)a.slots + j;
-                double acc[4] = {0, 0, 0, 0};
-                int b = wp;
-                for (; b + 3 * nw < a.nblk; b += 4 * nw) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) acc[u] += sl[(long long)(b + u * nw) * a.nobs];
-                }
-                for (; b < a.nblk; b += nw) acc[0] += sl[(long long)b * a.nobs];
-                sd[wp][lane] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                for (int u = 0; u < 4; ++u) acc[u] += (unsigned long long)sl[(long long)(b + u * nw) * a.nobs];
             }
+            for (; b < a.nblk; b += nw) acc[0] += (unsigned long long)sl[(long long)b * a.nobs];
+            si[wp][lane] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
         }
         __syncthreads();
         if (wp == 0 && j < a.nobs) {
-            if (a.fixed) {
-                unsigned long long tot = 0;
-                for (int k = 0; k < nw; ++k) tot += si[k][lane];
-                yv = (double)(long long)tot * a.q;
-            } else {
-                for (int k = 0; k < nw; ++k) yv += sd[k][lane];
-            }
+            unsigned long long tot = 0;
+            for (int k = 0; k < nw; ++k) tot += si[k][lane];
+            yv = (double)(long long)tot * a.q;
             have = true;
         }
     }

@@ -107,7 +107,6 @@ __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSme
     const bool need_cc = (FL & F_UPD) && cache_read;
     // 32-bit indices: n < 2^31, so i + stride stays below 2^32
     const unsigned n = (unsigned)a.n, stride = (unsigned)G * NT;
-    float emin = 0.f, emax = 0.f, lzm = 0.f;       // unused (FP32C range: shared-memory keys)
     unsigned i = ((threadIdx.x >> 5) * (unsigned)G + blockIdx.x) * 32u + (threadIdx.x & 31);
     float x = 0.f, y = 0.f, z = 0.f, vx = 0.f, vy = 0.f, vz = 0.f, wh = 0.f;
     double w = 0.0;
@@ -138,7 +137,7 @@ __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSme
             if (need_cc) ncc = *at(a.cell_cache, o4);
         }
         if (i < n) {
-            particle<float, L, FL, PK>(a, S, (int)i, x, y, z, vx, vy, vz, w, wh, cc, t, emin, emax, lzm, fs, epoch,
+            particle<float, L, FL, PK>(a, S, (int)i, x, y, z, vx, vy, vz, w, wh, cc, t, fs, epoch,
                                        cache_read);
             const size_t o4 = (size_t)i * 4u, o8 = (size_t)i * 8u;
             __stcs(at(px, o4), x); __stcs(at(py, o4), y); __stcs(at(pz, o4), z);
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
         if (s > 0 && b == G - 1 && wp == NT / 32 - 1)
             record_warp(A.chi2 + (size_t)3 * (par ^ 1) * G, G, A.st2 + (size_t)2 * (par ^ 1) * G, G, r.mu, A.t0 + s,
                         1, r.ring, r.last, a.err);
-        ThreadAcc t{0.0, 0.0, 0.f, 0.f, false, false};
+        ThreadAcc t{0.f, 0.f, false, false};
         if (upd) {
             if (rng) steps_particles<L, PK, F_STEADY | F_MINMAX>(a, S, G, nit, t, fs, epoch, cache_read);
             else steps_particles<L, PK, F_STEADY>(a, S, G, nit, t, fs, epoch, cache_read);
