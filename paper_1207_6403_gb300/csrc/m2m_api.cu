@@ -805,32 +805,15 @@ int sh_recompute(m2m_ctx *ctx) {
         CU(cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(512), args, sm, ctx->st));
     }
     const double q = ldexp(1.0, -a.sh);
-    const size_t tsm = ctx->sh_basis ? 8 * sh_sums(ctx) : 160 * (size_t)K;
-    if (ctx->sh_basis) {
-        LaunchTimer lt(ctx, M2M_TK_SH);
+    void *tab = ctx->sh_basis == 1 ? (f32 ? (void *)k_ex_tables<TriBasis, float> : (void *)k_ex_tables<TriBasis, double>)
+              : ctx->sh_basis == 2 ? (f32 ? (void *)k_ex_tables<FullBasis, float> : (void *)k_ex_tables<FullBasis, double>)
+                                   : (f32 ? (void *)k_sh_tables<float> : (void *)k_sh_tables<double>);
+    const int terms = ctx->sh_basis == 1 ? TriBasis::NT : ctx->sh_basis == 2 ? FullBasis::NT : 5;
+    {
         const long long *sum = (const long long *)ctx->d_sh_sum;
-        if (ctx->sh_basis == 1 && f32)
-            k_ex_tables<TriBasis, float><<<1, 512, tsm, ctx->st>>>(sum, K, ctx->d_sh_rnd, q, (float *)ctx->d_sh_tab,
-                                                                   ctx->d_err);
-        else if (ctx->sh_basis == 1)
-            k_ex_tables<TriBasis, double><<<1, 512, tsm, ctx->st>>>(sum, K, ctx->d_sh_rnd, q, (double *)ctx->d_sh_tab,
-                                                                    ctx->d_err);
-        else if (f32)
-            k_ex_tables<FullBasis, float><<<1, 512, tsm, ctx->st>>>(sum, K, ctx->d_sh_rnd, q, (float *)ctx->d_sh_tab,
-                                                                    ctx->d_err);
-        else
-            k_ex_tables<FullBasis, double><<<1, 512, tsm, ctx->st>>>(sum, K, ctx->d_sh_rnd, q,
-                                                                     (double *)ctx->d_sh_tab, ctx->d_err);
-        CU(cudaGetLastError());
-    } else {
+        void *args[] = {&sum, (void *)&ctx->sh_K, &ctx->d_sh_rnd, (void *)&q, &ctx->d_sh_tab, &ctx->d_err};
         LaunchTimer lt(ctx, M2M_TK_SH);
-        if (f32)
-            k_sh_tables<float><<<1, 256, tsm, ctx->st>>>((const long long *)ctx->d_sh_sum, K, ctx->d_sh_rnd, q,
-                                                         (float *)ctx->d_sh_tab, ctx->d_err);
-        else
-            k_sh_tables<double><<<1, 256, tsm, ctx->st>>>((const long long *)ctx->d_sh_sum, K, ctx->d_sh_rnd, q,
-                                                          (double *)ctx->d_sh_tab, ctx->d_err);
-        CU(cudaGetLastError());
+        CU(cudaLaunchKernel(tab, dim3(terms), dim3(256), args, 32 * (size_t)K, ctx->st));
     }
     return M2M_OK;
 }
@@ -1141,11 +1124,9 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     // the pass kernels may use more than 48 KB of shared memory
     const int optin = ctx->smem_optin;
     std::vector<void *> kfns = {cells_kernel_f32(), cells_kernel_f64(), (void *)k_sh_coef<float>,
-                                (void *)k_sh_coef<double>, (void *)k_sh_tables<float>, (void *)k_sh_tables<double>,
+                                (void *)k_sh_coef<double>,
                                 (void *)k_ex_coef<TriBasis, float>, (void *)k_ex_coef<TriBasis, double>,
-                                (void *)k_ex_tables<TriBasis, float>, (void *)k_ex_tables<TriBasis, double>,
-                                (void *)k_ex_coef<FullBasis, float>, (void *)k_ex_coef<FullBasis, double>,
-                                (void *)k_ex_tables<FullBasis, float>, (void *)k_ex_tables<FullBasis, double>};
+                                (void *)k_ex_coef<FullBasis, float>, (void *)k_ex_coef<FullBasis, double>};
     for (int lay = 0; lay < 5; ++lay) {
         for (int nt : {256, 512, 1024}) kfns.push_back(pass_kernel_f32(nt, lay));
         for (int nt : {256, 512}) kfns.push_back(pass_kernel_f64(nt, lay));

@@ -1433,19 +1433,18 @@ __global__ void __launch_bounds__(512) k_sh_coef(const __grid_constant__ ShArgs 
     if (bad) atomicOr(a.err, ERR_NONFINITE);
 }
 
-// Node tables from the side sums (one block): scale back, prefix sums for
-// A_l(r_k) = sum_{j <= k}, suffix sums (outside in) for B_l(r_k) =
-// sum_{j > k}, then F_l, D_l and the slopes to the next node, in double.
+// Node sums of one term from its side sums (one block): scaled back to r_j^l
+// and r_(j-1)^-(l+1), then A(r_k) = sum_{j <= k} by a prefix and B(r_k) =
+// sum_{j > k} by a suffix sum (outside in), each in order by one thread; S:
+// [2][K], row 0 from rowA of the side sums, row 1 from rowB.
 template <class R>
-__global__ void k_sh_tables(const long long *sum, int K, const double *rn, double q, R *tab, int *err) {
-    extern __shared__ __align__(16) double sd[];
-    double *S = sd;                // [10][K] side sums, then A, B at the nodes
-    double *FD = sd + 10 * K;      // [10][K] F_l, D_l at the nodes
-    for (int k = threadIdx.x; k < 10 * K; k += blockDim.x) {
-        const int m = k / K, j = k - m * K, n = m % 5, l = 2 * n;
-        const double v = sizeof(R) == 4 ? (double)sum[k] * q : ((const double *)sum)[k];
+__device__ __forceinline__ void node_sums(const long long *sum, int rowA, int rowB, int l, int K, const double *rn,
+                                          double q, double *S) {
+    for (int k = threadIdx.x; k < 2 * K; k += blockDim.x) {
+        const int side = k / K, j = k - side * K, at = (side ? rowB : rowA) * K + j;
+        const double v = sizeof(R) == 4 ? (double)sum[at] * q : ((const double *)sum)[at];
         double s = 1.0;
-        if (m < 5) {
+        if (side == 0) {
             for (int e = 0; e < l; ++e) s *= rn[j];                       // r_j^l
         } else if (j > 0) {
             for (int e = 0; e <= l; ++e) s *= rn[j - 1];                  // r_(j-1)^(l+1)
@@ -1456,42 +1455,46 @@ __global__ void k_sh_tables(const long long *sum, int K, const double *rn, doubl
         S[k] = v * s;
     }
     __syncthreads();
-    if (threadIdx.x < 10) {
-        double *row = S + threadIdx.x * K;
-        double acc = 0.0;
-        if (threadIdx.x < 5) {
-            for (int k = 0; k < K; ++k) { acc += row[k]; row[k] = acc; }
-        } else {
-            for (int k = K - 1; k >= 0; --k) { const double b = row[k]; row[k] = acc; acc += b; }
-        }
+    double acc = 0.0;
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < K; ++k) { acc += S[k]; S[k] = acc; }
+    } else if (threadIdx.x == 32) {
+        for (int k = K - 1; k >= 0; --k) { const double b = S[K + k]; S[K + k] = acc; acc += b; }
     }
     __syncthreads();
+}
+
+// Node table of the axisymmetric expansion, one block per l: F_l, D_l and the
+// slopes to the next node, in double.  (One block for all of them kept a
+// single SM busy with some 50 FP64 operations per node and term: 52 us for
+// 256 nodes, 12 now; the triaxial table 145, 14 now.)
+template <class R>
+__global__ void __launch_bounds__(256) k_sh_tables(const long long *sum, int K, const double *rn, double q, R *tab,
+                                                   int *err) {
+    extern __shared__ __align__(16) double sd[];
+    const int n = blockIdx.x, l = 2 * n;
+    double *F = sd + 2 * K, *D = sd + 3 * K;
+    node_sums<R>(sum, n, 5 + n, l, K, rn, q, sd);
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const double r = rn[k], ir = 1.0 / r;
         double rl = 1.0;           // r^l
-        for (int n = 0; n < 5; ++n) {
-            const int l = 2 * n;
-            const double A = S[n * K + k], B = S[(5 + n) * K + k];
-            const double irl1 = ir / rl;                  // r^-(l+1)
-            FD[n * K + k] = A * irl1 + B * rl;
-            FD[(5 + n) * K + k] = -(double)(l + 1) * A * (irl1 * ir) + (l > 0 ? (double)l * B * (rl * ir) : 0.0);
-            rl = rl * r * r;
-        }
-        if (!isfinite(FD[k])) atomicOr(err, ERR_NONFINITE);
+        for (int e = 0; e < n; ++e) rl = rl * r * r;
+        const double A = sd[k], B = sd[K + k];
+        const double irl1 = ir / rl;                  // r^-(l+1)
+        F[k] = A * irl1 + B * rl;
+        D[k] = -(double)(l + 1) * A * (irl1 * ir) + (l > 0 ? (double)l * B * (rl * ir) : 0.0);
+        if (n == 0 && !isfinite(F[k])) atomicOr(err, ERR_NONFINITE);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         R *row = tab + (size_t)k * SH_ROW;
         const bool last = k == K - 1;
         const double h = last ? 1.0 : 1.0 / (rn[k + 1] - rn[k]);
-        for (int n = 0; n < 5; ++n) {
-            const double F = FD[n * K + k], D = FD[(5 + n) * K + k];
-            row[n] = (R)F;
-            row[10 + n] = (R)D;
-            row[5 + n] = last ? R(0) : (R)((FD[n * K + k + 1] - F) * h);
-            row[15 + n] = last ? R(0) : (R)((FD[(5 + n) * K + k + 1] - D) * h);
-        }
-        row[20] = (R)rn[k];
+        row[n] = (R)F[k];
+        row[10 + n] = (R)D[k];
+        row[5 + n] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
+        row[15 + n] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
+        if (n == 0) row[20] = (R)rn[k];
     }
 }
 
@@ -1599,73 +1602,38 @@ __global__ void __launch_bounds__(512) k_ex_coef(const __grid_constant__ ShArgs 
     if (bad) atomicOr(a.err, ERR_NONFINITE);
 }
 
-// F_t and D_t at node k from the node sums A (rows 0..NT-1) and B (rows
-// NT..2NT-1) held in S ([2NT][K]), with the 4 pi/(2l+1) of the addition
-// theorem.
-template <class B>
-__device__ __forceinline__ void ex_node_FD(const double *S, int K, const double *rn, int k, int t, double &F,
-                                           double &D) {
-    const int l = B::l_of(t);
-    const double r = rn[k], ir = 1.0 / r;
-    double rl = 1.0;
-    for (int e = 0; e < l; ++e) rl *= r;                           // r^l
-    const double A = S[t * K + k], Bs = S[(B::NT + t) * K + k];
-    const double c = 12.566370614359172 / (double)(2 * l + 1);     // 4 pi/(2l+1)
-    const double irl1 = ir / rl;                                   // r^-(l+1)
-    F = c * (A * irl1 + Bs * rl);
-    D = c * (-(double)(l + 1) * A * (irl1 * ir) + (l > 0 ? (double)l * Bs * (rl * ir) : 0.0));
-}
-
-// Node tables of an expansion with m != 0 from its side sums (one block):
-// scale back, prefix sums (A) and suffix sums (B), then F_t, D_t and the
-// slopes to the next node.
+// Node table of an expansion with m != 0, one block per term t: F_t and D_t
+// with the 4 pi/(2l+1) of the addition theorem, then the slopes to the next
+// node.
 template <class B, class R>
-__global__ void k_ex_tables(const long long *sum, int K, const double *rn, double q, R *tab, int *err) {
+__global__ void __launch_bounds__(256) k_ex_tables(const long long *sum, int K, const double *rn, double q, R *tab,
+                                                   int *err) {
     extern __shared__ __align__(16) double sd[];
-    constexpr int NT = B::NT, NR = 2 * NT, ROW = B::ROW;
-    double *S = sd;                // [2NT][K] side sums, then A, B at the nodes
-    for (int k = threadIdx.x; k < NR * K; k += blockDim.x) {
-        const int row = k / K, j = k - row * K, t = row % NT, l = B::l_of(t);
-        const double v = sizeof(R) == 4 ? (double)sum[k] * q : ((const double *)sum)[k];
-        double s = 1.0;
-        if (row < NT) {
-            for (int e = 0; e < l; ++e) s *= rn[j];                       // r_j^l
-        } else if (j > 0) {
-            for (int e = 0; e <= l; ++e) s *= rn[j - 1];                  // r_(j-1)^(l+1)
-            s = 1.0 / s;
-        } else {
-            s = 0.0;
-        }
-        S[k] = v * s;
-    }
-    __syncthreads();
-    if (threadIdx.x < NR) {
-        double *row = S + threadIdx.x * K;
-        double acc = 0.0;
-        if (threadIdx.x < NT) {
-            for (int k = 0; k < K; ++k) { acc += row[k]; row[k] = acc; }
-        } else {
-            for (int k = K - 1; k >= 0; --k) { const double b = row[k]; row[k] = acc; acc += b; }
-        }
+    constexpr int NT = B::NT, ROW = B::ROW;
+    const int t = blockIdx.x, l = B::l_of(t);
+    double *F = sd + 2 * K, *D = sd + 3 * K;
+    node_sums<R>(sum, t, NT + t, l, K, rn, q, sd);
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const double r = rn[k], ir = 1.0 / r;
+        double rl = 1.0;
+        for (int e = 0; e < l; ++e) rl *= r;                           // r^l
+        const double A = sd[k], Bs = sd[K + k];
+        const double c = 12.566370614359172 / (double)(2 * l + 1);     // 4 pi/(2l+1)
+        const double irl1 = ir / rl;                                   // r^-(l+1)
+        F[k] = c * (A * irl1 + Bs * rl);
+        D[k] = c * (-(double)(l + 1) * A * (irl1 * ir) + (l > 0 ? (double)l * Bs * (rl * ir) : 0.0));
+        if (!(isfinite(F[k]) && isfinite(D[k]))) atomicOr(err, ERR_NONFINITE);
     }
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         R *row = tab + (size_t)k * ROW;
         const bool last = k == K - 1;
         const double h = last ? 1.0 : 1.0 / (rn[k + 1] - rn[k]);
-        bool fin = true;
-        for (int t = 0; t < NT; ++t) {
-            double F, D, F1 = 0.0, D1 = 0.0;
-            ex_node_FD<B>(S, K, rn, k, t, F, D);
-            if (!last) ex_node_FD<B>(S, K, rn, k + 1, t, F1, D1);
-            fin = fin && isfinite(F) && isfinite(D);
-            row[t] = (R)F;
-            row[2 * NT + t] = (R)D;
-            row[NT + t] = last ? R(0) : (R)((F1 - F) * h);
-            row[3 * NT + t] = last ? R(0) : (R)((D1 - D) * h);
-        }
-        row[4 * NT] = (R)rn[k];
-        if (!fin) atomicOr(err, ERR_NONFINITE);
+        row[t] = (R)F[k];
+        row[2 * NT + t] = (R)D[k];
+        row[NT + t] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
+        row[3 * NT + t] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
+        if (t == 0) row[4 * NT] = (R)rn[k];
     }
 }
 
