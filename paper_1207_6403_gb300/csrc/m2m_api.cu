@@ -1031,7 +1031,7 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     if (!f32) ALLOC(ctx->d_exp, 8 * EXP_N);
     ALLOC(ctx->d_y_acc, (size_t)8 * nobs);
     ALLOC(ctx->d_stat_slots, (size_t)32 * ctx->slot_cap);
-    ALLOC(ctx->d_rec_ticket, 8);
+    ALLOC(ctx->d_rec_ticket, 16);              // a context's own passes, batched passes
     ALLOC(ctx->d_chi_slots, (size_t)24 * ((nobs + 31) / 32 + 1));
     ALLOC(ctx->d_bar, 8);
     ALLOC(ctx->d_st2, (size_t)32 * ctx->slot_cap);
@@ -1087,7 +1087,7 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         if (e4 == cudaSuccess) e4 = cudaMemcpy(ctx->d_isig, isig.data(), 8 * nobs, cudaMemcpyHostToDevice);
         cudaError_t e5 = cudaMemset(ctx->d_Dt, 0, 8 * nobs);
         cudaError_t e6 = cudaMemset(ctx->d_ticket, 0, 4);
-        if (e6 == cudaSuccess) e6 = cudaMemset(ctx->d_rec_ticket, 0, 8);
+        if (e6 == cudaSuccess) e6 = cudaMemset(ctx->d_rec_ticket, 0, 16);
         cudaError_t e7 = cudaMemset(ctx->d_err, 0, 4);
         cudaError_t e8 = cudaMemset(ctx->d_coef_r, 0, rs * nobs);
         cudaError_t e9 = cudaMemset(ctx->d_ring, 0, sizeof(m2m_record) * M2M_HISTORY);
@@ -1839,10 +1839,14 @@ struct m2m_batch {
     int period = 0;              // common moving-prior period (0: flat)
     PassArgs *d_pass = nullptr;  // per-model arguments
     ResArgs *d_res = nullptr;
-    int *d_tab = nullptr;        // pass: model, rank, count | residual: model, rank, count
+    int *d_tab = nullptr;        // residual: model, rank, count | pass: first segment of a block, segments of a
+                                 // model, segments
     int pgrid = 0, rgrid = 0;
     int mult = 1;                // pass blocks = mult * SMs * resident blocks (autotuned)
-    std::vector<int> pcount, rcount;
+    std::vector<int> pcount, rcount;   // pass segments and residual blocks of each model
+    std::vector<PassArgs> up_pass;     // what the device arrays hold
+    std::vector<ResArgs> up_res;
+    long long up_step = -1;            // and the device step counter
     long long *d_step = nullptr; // step counter read by the batched residual
     void *d_gather = nullptr;    // record gather: source pointers, records, error words
     long long t = 0;
@@ -1888,6 +1892,11 @@ int batch_upload(m2m_batch *b) {
         if (rc) return berr(b, rc, "model %d record: %s", m, c->err.c_str());
         c->stat_par = 0;
         fill_args(c, pa[m], 0);
+        pa[m].rec_chi_nblk = b->rcount[m];
+        pa[m].rec_stat_nblk = b->pcount[m];
+        pa[m].rec_ticket = c->d_rec_ticket + 1;
+        pa[m].rec_base = 0;
+        pa[m].epoch = 0;                     // unused: a fused batch has no seeing
         ResArgs &r = ra[m];
         memset(&r, 0, sizeof r);
         r.slots = c->d_slots; r.nblk = b->pcount[m]; r.nobs = c->nobs; r.y_acc = c->d_y_acc;
@@ -1901,11 +1910,19 @@ int batch_upload(m2m_batch *b) {
         r.tail = 1;
         r.err = c->d_err;
     }
+    if (b->up_pass.size() == pa.size() && b->up_res.size() == ra.size() &&
+        !memcmp(b->up_pass.data(), pa.data(), sizeof(PassArgs) * pa.size()) &&
+        !memcmp(b->up_res.data(), ra.data(), sizeof(ResArgs) * ra.size()))
+        return M2M_OK;                       // the device holds these already
+    b->up_pass.clear();
+    b->up_res.clear();
     cudaError_t e = cudaMemcpyAsync(b->d_pass, pa.data(), sizeof(PassArgs) * b->nmodels, cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->d_res, ra.data(), sizeof(ResArgs) * b->nmodels, cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);   // host staging buffers go out of scope
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "batch upload: %s", cudaGetErrorString(e));
+    b->up_pass.swap(pa);
+    b->up_res.swap(ra);
     return M2M_OK;
 }
 
@@ -1915,32 +1932,43 @@ size_t batch_smem(const m2m_batch *b, int flags) {
     return sm;
 }
 
-int batch_pass(m2m_batch *b, int flags, int cache_read) {
+// half: of the S, sum w partials; rec_step > 0: also writes the record of
+// step *d_step + rec_step, whose residual left its partials
+int batch_pass(m2m_batch *b, int flags, int cache_read, int half, long long rec_step) {
     BatchPass bp;
     bp.models = b->d_pass;
-    bp.blk_model = b->d_tab;
-    bp.blk_rank = b->d_tab + b->pgrid;
-    bp.blk_count = b->d_tab + 2 * b->pgrid;
+    bp.blk_seg = b->d_tab + 2 * b->rgrid + b->nmodels;        // see batch_plan
+    bp.model_segs = bp.blk_seg + b->pgrid + 1;
+    bp.segs = (const BatchSeg *)(bp.model_segs + b->nmodels);
     bp.flags = flags;
     bp.cache_read = cache_read;
     bp.cache_write = 1;
+    bp.half = half;
+    bp.slot_cap = b->ctx[0]->slot_cap;
+    bp.rec = rec_step > 0;
+    bp.rec_step = rec_step;
+    bp.step = b->d_step;
     void *args[] = {&bp};
     const bool steady = flags == F_STEADY && cache_read;
-    cudaError_t e = cudaLaunchKernel(pass_kernel_f32_batch(b->layout, steady, b->pk), dim3(b->pgrid), dim3(1024), args,
+    cudaError_t e = launch_dependent(pass_kernel_f32_batch(b->layout, steady, b->pk), dim3(b->pgrid), dim3(1024), args,
                                      batch_smem(b, flags), b->st);
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "batched pass: %s", cudaGetErrorString(e));
     return M2M_OK;
 }
 
 // One fused step sequence of nsteps steps starting at step t0 with the
-// models' update pending or not.  Records are numbered from *d_step.
+// models' update pending or not.  Records are numbered from *d_step; a
+// step's record is written by the pass that follows its residual (by the
+// residual itself where none does).
 int batch_sequence(m2m_batch *b, long long nsteps, long long t0, bool pending) {
-    const int *rtab = b->d_tab + 2 * b->pgrid + b->nmodels;   // see the table layout in m2m_batch_init
+    const int *rtab = b->d_tab;               // see the table layout in batch_plan
+    long long rec = 0;                        // relative step of the record left to the next pass
     for (long long k = 0; k < nsteps; ++k) {
         const long long t1 = t0 + k + 1;
+        const int half = (int)(k & 1);
         const bool prior_due = b->period > 0 && (t1 % b->period == 0);
         int fl = F_PUSH | F_SCAT | F_STATS | (pending ? F_UPD : 0) | (prior_due ? F_MINMAX : 0);
-        int rc = batch_pass(b, fl, pending ? 1 : 0);
+        int rc = batch_pass(b, fl, pending ? 1 : 0, half, rec);
         if (rc) return rc;
         BatchRes br;
         br.models = b->d_res;
@@ -1949,10 +1977,14 @@ int batch_sequence(m2m_batch *b, long long nsteps, long long t0, bool pending) {
         br.blk_count = rtab + 2 * b->rgrid;
         br.mode = 1;
         br.write_ring = 1;
+        br.tail = prior_due ? 1 : 0;
+        br.half = half;
+        br.slot_cap = b->ctx[0]->slot_cap;
         br.rec_step = (long long)(k + 1);     // relative: k_residual_batch adds *d_step
         br.step = b->d_step;
+        rec = prior_due ? 0 : k + 1;
         void *args[] = {&br};
-        cudaError_t e = cudaLaunchKernel((void *)k_residual_batch, dim3(b->rgrid), dim3(RES_NT_FX), args, 0, b->st);
+        cudaError_t e = launch_dependent((void *)k_residual_batch, dim3(b->rgrid), dim3(RES_NT_FX), args, 0, b->st);
         if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "batched residual: %s", cudaGetErrorString(e));
         pending = true;
         if (prior_due) {
@@ -1966,7 +1998,7 @@ int batch_sequence(m2m_batch *b, long long nsteps, long long t0, bool pending) {
         }
     }
     if (pending) {
-        int rc = batch_pass(b, F_UPD, 1);
+        int rc = batch_pass(b, F_UPD, 1, (int)(nsteps & 1), rec);
         if (rc) return rc;
     }
     k_add_step<<<1, 1, 0, b->st>>>(b->d_step, nsteps);
@@ -1976,10 +2008,15 @@ int batch_sequence(m2m_batch *b, long long nsteps, long long t0, bool pending) {
 }
 
 // Block plan of the fused batch: mult * (SMs x resident blocks) pass blocks
-// in proportion to N_m (at least one per model, largest remainders first),
-// one residual block per 128 observables of each model; device tables
-// [model | rank | count] for the pass, then for the residual.  Drops the
-// captured graphs (their launch shapes change).
+// that each take the same work from the models' particles laid end to end, a
+// model's part of a block being a segment; a segment counts SEG_COST
+// particles beside its own (its tables and its histogram's clearing and flush
+// take about 6 us of a block, as 2000 particles do).  One residual block per 128
+// observables of each model.  Device tables: residual [model(rgrid) |
+// rank(rgrid) | count(nmodels)], pass [first segment(pgrid + 1) |
+// segments(nmodels) | segments].  Drops the captured graphs (their launch
+// shapes change).
+constexpr long long SEG_COST = 2000;
 int batch_plan(m2m_batch *b, int mult) {
     for (auto &g : b->graphs) cudaGraphExecDestroy(g.second);
     b->graphs.clear();
@@ -1993,50 +2030,67 @@ int batch_plan(m2m_batch *b, int mult) {
         g_init_error = "batched pass does not fit";
         return M2M_OK;
     }
-    long long G = (long long)c0->nsm * occ * mult;
-    double tot = 0;
-    for (m2m_ctx *c : b->ctx) tot += (double)c->n;
-    std::vector<double> share(nmodels);
-    int used = 0;
-    b->pcount.assign(nmodels, 1);
-    for (int m = 0; m < nmodels; ++m) {
-        share[m] = G * (double)b->ctx[m]->n / tot;
-        b->pcount[m] = std::max(1, (int)share[m]);
-        long long need = (b->ctx[m]->n + 1023) / 1024;
-        b->pcount[m] = (int)std::min<long long>(std::min<long long>(b->pcount[m], need), b->ctx[m]->slot_cap);
-        used += b->pcount[m];
-    }
-    for (int extra = (int)G - used; extra > 0; --extra) {     // largest remainders first
-        int best = -1;
-        double bestr = 0;
+    // segments by filling each block up to a level of work; the lowest level
+    // that needs at most G blocks, by bisection
+    const long long G = (long long)c0->nsm * occ * mult;
+    std::vector<BatchSeg> segs;
+    std::vector<int> first;
+    auto fill = [&](long long level) {
+        segs.clear();
+        first.assign(1, 0);
+        b->pcount.assign(nmodels, 0);
+        long long room = level;
         for (int m = 0; m < nmodels; ++m) {
-            long long need = (b->ctx[m]->n + 1023) / 1024;
-            if (b->pcount[m] >= need || b->pcount[m] >= b->ctx[m]->slot_cap) continue;
-            double r = share[m] - b->pcount[m];
-            if (best < 0 || r > bestr) { best = m; bestr = r; }
+            long long at = 0;
+            while (at < b->ctx[m]->n) {
+                if (room < SEG_COST + 1024 && room < level) {    // too little left for a segment: next block
+                    first.push_back((int)segs.size());
+                    room = level;
+                }
+                // whole warps, so that every segment starts on a 128-byte line
+                long long take = ((room - SEG_COST) / 32) * 32;
+                // the rest of the model where it fits, or where its slots are used up
+                if (take >= b->ctx[m]->n - at || b->pcount[m] == c0->slot_cap - 1) take = b->ctx[m]->n - at;
+                segs.push_back({m, b->pcount[m]++, (int)at, (int)(at + take)});
+                at += take;
+                room -= take + SEG_COST;
+            }
         }
-        if (best < 0) break;
-        ++b->pcount[best];
+        first.push_back((int)segs.size());
+        return (long long)first.size() - 1 <= G;
+    };
+    long long total = 0;
+    for (m2m_ctx *c : b->ctx) total += c->n + SEG_COST;
+    long long lo = SEG_COST + 1024, hi = total + SEG_COST + 1024;    // hi: one block does it all
+    if (fill(lo)) hi = lo;
+    while (hi - lo > 32) {
+        const long long mid = (lo + hi) / 2;
+        if (fill(mid)) hi = mid; else lo = mid;
     }
+    fill(hi);
+    b->pgrid = (int)first.size() - 1;
     b->rcount.assign(nmodels, 1);
     for (int m = 0; m < nmodels; ++m) b->rcount[m] = (b->ctx[m]->nobs + RES_NT_FX - 1) / RES_NT_FX;
-    b->pgrid = 0;
-    for (int m = 0; m < nmodels; ++m) b->pgrid += b->pcount[m];
     b->rgrid = 0;
     for (int m = 0; m < nmodels; ++m) b->rgrid += b->rcount[m];
-    std::vector<int> tab, pm_, pr_, rm_, rr_;
-    for (int m = 0; m < nmodels; ++m)
-        for (int k = 0; k < b->pcount[m]; ++k) { pm_.push_back(m); pr_.push_back(k); }
+    std::vector<int> tab, rm_, rr_;
     for (int m = 0; m < nmodels; ++m)
         for (int k = 0; k < b->rcount[m]; ++k) { rm_.push_back(m); rr_.push_back(k); }
-    tab.insert(tab.end(), pm_.begin(), pm_.end());
-    tab.insert(tab.end(), pr_.begin(), pr_.end());
-    tab.insert(tab.end(), b->pcount.begin(), b->pcount.end());
     tab.insert(tab.end(), rm_.begin(), rm_.end());
     tab.insert(tab.end(), rr_.begin(), rr_.end());
     tab.insert(tab.end(), b->rcount.begin(), b->rcount.end());
-    // table layout: pass [model(pgrid) | rank(pgrid) | count(nmodels)],
-    // then residual [model(rgrid) | rank(rgrid) | count(nmodels)]
+    tab.insert(tab.end(), first.begin(), first.end());
+    tab.insert(tab.end(), b->pcount.begin(), b->pcount.end());
+    for (const BatchSeg &q : segs) {
+        const int v[] = {q.model, q.rank, q.begin, q.end};
+        tab.insert(tab.end(), v, v + 4);
+    }
+    b->up_pass.clear();               // the segment counts are part of the arguments
+    for (m2m_ctx *c : b->ctx)         // REC_EVERY counts from a multiple of the segments
+        if (cudaMemsetAsync(c->d_rec_ticket + 1, 0, 8, b->st) != cudaSuccess) {
+            g_init_error = "record ticket reset";
+            return M2M_ERR_CUDA;
+        }
     if (b->d_tab) { cudaFree(b->d_tab); b->d_tab = nullptr; }
     e = cudaMalloc(&b->d_tab, sizeof(int) * tab.size());
     if (e == cudaSuccess) e = cudaMemcpy(b->d_tab, tab.data(), sizeof(int) * tab.size(), cudaMemcpyHostToDevice);
@@ -2139,8 +2193,12 @@ int m2m_batch_step(m2m_batch *b, int64_t nsteps) {
     if (rc) return rc;
     // step counter of the records: the models' common step count
     long long t0 = b->ctx[0]->t;
-    cudaError_t e = cudaMemcpyAsync(b->d_step, &t0, sizeof t0, cudaMemcpyHostToDevice, b->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
+    cudaError_t e = cudaSuccess;
+    if (b->up_step != t0) {
+        e = cudaMemcpyAsync(b->d_step, &t0, sizeof t0, cudaMemcpyHostToDevice, b->st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
+    }
+    b->up_step = -1;
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "step counter: %s", cudaGetErrorString(e));
     const bool graphable = b->st != nullptr && b->st != cudaStreamLegacy && b->st != cudaStreamPerThread;
     const auto key = std::make_tuple((long long)nsteps, b->period ? t0 % b->period : 0ll, 0);
@@ -2182,6 +2240,7 @@ int m2m_batch_step(m2m_batch *b, int64_t nsteps) {
         if (rc) return rc;
         b->last_mode = 1;
     }
+    b->up_step = t0 + nsteps;                // k_add_step advances it
     for (int m = 0; m < b->nmodels; ++m) {
         m2m_ctx *c = b->ctx[m];
         c->t = t0 + nsteps;

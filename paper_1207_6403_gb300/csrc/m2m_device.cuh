@@ -20,6 +20,7 @@ constexpr int MAXCELLS = 16385;
 
 enum { F_UPD = 1, F_PUSH = 2, F_SCAT = 4, F_STATS = 8, F_MINMAX = 16, F_CELLS = 32 };
 enum { G_LIN = 0, G_LOG = 1, G_BIS = 2 };
+enum { REC_EVERY = 2 };
 enum { C64_LNW = 1, C64_GH = 2 };
 enum { ERR_NONFINITE = 1, ERR_OVERFLOW = 2, ERR_TIMEOUT = 4 };
 
@@ -99,6 +100,7 @@ struct PassArgs {
     void *facc; int facc_read;              // expansion potentials: force at the positions (R, [3][n]) or NULL
     // record of the preceding step, left by its residual to this pass (the
     // first block to finish its particles writes it; see record_warp)
+    // (rec_pending REC_EVERY: each launch of nblk tickets has a record to write)
     int rec_pending, rec_write_ring, rec_chi_nblk, rec_stat_nblk;
     long long rec_step;
     unsigned long long rec_base;            // rec_ticket value the first block sees
