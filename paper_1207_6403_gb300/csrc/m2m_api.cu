@@ -250,7 +250,8 @@ size_t pass_smem_copies(const m2m_ctx *c, int flags, int hrep) {
 // of 4.1M particles in all, 25 steps, 4.17 / 4.07 / 3.99 ms; 1M particles,
 // 25 steps, 774 / 767 / 777 us.
 int hist_copies(const m2m_ctx *c) {
-    const size_t room = (size_t)c->smem_optin - 4096;       // the kernels' static shared memory
+    // the kernels' static shared memory, and a solo residual's arrays
+    const size_t room = (size_t)c->smem_optin - 4096 - (c->nobs <= SOLO_OBS ? 16 * (size_t)c->nobs : 0);
     if (c->prec == M2M_FP32C && (c->threads != 1024 || c->pipe || (c->layout != 2 && c->layout != 3))) return 1;
     int r = c->launch_n >= 8ll * 1024 * c->nsm ? 32 : 8;
     if (c->prec == M2M_FP64) {
@@ -543,17 +544,24 @@ int prior_recompute(m2m_ctx *ctx, int pass_flags) {
     return M2M_OK;
 }
 
-// The persistent multi-step kernel for this context, or NULL where it does
+// The persistent multi-step kernel for m steps of this context, or NULL where it does
 // not apply (FP64, the run-time set walk, the spherical-harmonic potential,
 // the bulk-copy pipeline or per-block histogram slots chosen, a potential
 // signature without one, or no room for one block per SM).
-void *persistent_kernel(m2m_ctx *ctx, size_t *smem_out, int *grid_out) {
+void *persistent_kernel(m2m_ctx *ctx, long long m, size_t *smem_out, int *grid_out, bool *solo_out) {
     if (!ctx->persist || ctx->prec != M2M_FP32C || ctx->layout == 0 || ctx->sh_on || ctx->pipe || !ctx->fx_atomic ||
         ctx->threads != 1024)
         return nullptr;
-    void *fn = steps_kernel_f32(ctx->layout, potential_signature(ctx));
+    void *fn = steps_kernel_f32(ctx->layout, potential_signature(ctx), false);
     if (!fn) return nullptr;
-    const size_t sm = pass_smem(ctx, F_STEADY);
+    size_t sm = pass_smem(ctx, F_STEADY);
+    *solo_out = false;
+    if (m >= 3 && ctx->nobs <= SOLO_OBS && sm + 16 * (size_t)ctx->nobs + 4096 <= (size_t)ctx->smem_optin)
+        if (void *fs = steps_kernel_f32(ctx->layout, potential_signature(ctx), true)) {
+            fn = fs;
+            sm += 16 * (size_t)ctx->nobs;
+            *solo_out = true;
+        }
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 1024, sm) != cudaSuccess || occ < 1) {
         cudaGetLastError();
@@ -571,7 +579,7 @@ void *persistent_kernel(m2m_ctx *ctx, size_t *smem_out, int *grid_out) {
 // m steps in one cooperative launch; the last takes the (E, L_z) range when
 // last_range.  Leaves the last step's weight update pending and its record
 // written.
-int launch_steps(m2m_ctx *ctx, void *fn, size_t sm, int grid, long long m, bool last_range) {
+int launch_steps(m2m_ctx *ctx, void *fn, size_t sm, int grid, bool solo, long long m, bool last_range) {
     int rc0 = finish_record(ctx);
     if (rc0) return rc0;
     StepsArgs A;
@@ -597,7 +605,8 @@ int launch_steps(m2m_ctx *ctx, void *fn, size_t sm, int grid, long long m, bool 
     A.wait_ns = ctx->test_stall ? ctx->test_wait_ns : ctx->wait_ns;
     A.test_stall = ctx->test_stall;
     ctx->test_stall = 0;
-    CU(cudaMemsetAsync(ctx->d_bar, 0, 8, ctx->st));
+    A.tot3 = solo ? ctx->d_bar + 1 : nullptr;
+    CU(cudaMemsetAsync(ctx->d_bar, 0, 8 + (solo ? 24 * (size_t)ctx->nobs : 0), ctx->st));
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3((unsigned)grid);
@@ -1033,7 +1042,7 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     ALLOC(ctx->d_stat_slots, (size_t)32 * ctx->slot_cap);
     ALLOC(ctx->d_rec_ticket, 16);              // a context's own passes, batched passes
     ALLOC(ctx->d_chi_slots, (size_t)24 * ((nobs + 31) / 32 + 1));
-    ALLOC(ctx->d_bar, 8);
+    ALLOC(ctx->d_bar, 8 + (nobs <= SOLO_OBS ? 24 * (size_t)nobs : 0));   // barrier, a solo residual's totals
     ALLOC(ctx->d_st2, (size_t)32 * ctx->slot_cap);
     ALLOC(ctx->d_chi2, (size_t)48 * ctx->slot_cap);
     ALLOC(ctx->d_ticket, 4);
@@ -1139,7 +1148,8 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         kfns.push_back(pass_kernel_f32_batch(lay));
         if (lay) kfns.push_back(pass_kernel_f32_batch(lay, true));
         if (lay == 2) kfns.push_back(pass_kernel_f32_batch(lay, true, PK_HERNQUIST_NFW));
-        for (int pk : {PK_HERNQUIST, PK_LOG, PK_HERNQUIST_NFW}) kfns.push_back(steps_kernel_f32(lay, pk));
+        for (int pk : {PK_HERNQUIST, PK_LOG, PK_HERNQUIST_NFW})
+            for (bool solo : {false, true}) kfns.push_back(steps_kernel_f32(lay, pk, solo));
     }
     for (void *f : kfns) {
         if (!f) continue;                    // no such variant compiled
@@ -1289,15 +1299,16 @@ static int run_steps(m2m_ctx *ctx, int64_t nsteps) {
         long long t1 = ctx->t + 1;
         size_t psm = 0;
         int pgrid = 0;
-        if (void *pf = persistent_kernel(ctx, &psm, &pgrid)) {
-            // the steps up to the next prior recompute (inclusive) in one launch
-            long long m = nsteps - k;
-            if (moving) {
-                const long long due = ((t1 + ctx->prior.period - 1) / ctx->prior.period) * ctx->prior.period;
-                if (due - t1 + 1 < m) m = due - t1 + 1;
-            }
+        bool solo = false;
+        // the steps up to the next prior recompute (inclusive) in one launch
+        long long m = nsteps - k;
+        if (moving) {
+            const long long due = ((t1 + ctx->prior.period - 1) / ctx->prior.period) * ctx->prior.period;
+            if (due - t1 + 1 < m) m = due - t1 + 1;
+        }
+        if (void *pf = persistent_kernel(ctx, m, &psm, &pgrid, &solo)) {
             const bool range = moving && ((t1 + m - 1) % ctx->prior.period == 0);
-            int rc = launch_steps(ctx, pf, psm, pgrid, m, range);
+            int rc = launch_steps(ctx, pf, psm, pgrid, solo, m, range);
             if (rc) return rc;
             if (range) {
                 rc = prior_recompute(ctx, F_UPD);

@@ -205,32 +205,14 @@ __device__ __forceinline__ int prior_cell(R x, R y, R z, R vx, R vy, R vz, const
 }
 
 // ----------------------------------------------------------------- record
-// The step record from the residual's per-block partials (chi^2, sum of
-// Delta^2, max |Delta~|: 3 doubles per block) and the pass's per-block
-// partials (S, sum w: 2 doubles per block), reduced by one warp in a fixed
-// order (lane k takes blocks k, k+32, ... in turn, then a fixed shuffle
-// tree): the same record whichever kernel computes it.  Lane 0 writes it.
-__device__ __forceinline__ void record_warp(const double *chi, int nch, const double *st, int nst, double mu,
-                                            long long step, int write_ring, m2m_record *ring, m2m_record *last,
-                                            int *err) {
-    const int lane = threadIdx.x & 31;
-    double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0;
-    // up to 8 partials per lane loaded before any is added (one memory
-    // latency instead of eight), then added in block order
+// The rest of record_warp: the lanes' chi^2 partials v0, v1 (sums) and v2
+// (maximum) with the per-block S, sum w partials, and lane 0's write.
+__device__ __forceinline__ void record_finish(double v0, double v1, double v2, const double *st, int nst, double mu,
+                                              long long step, int write_ring, m2m_record *ring, m2m_record *last,
+                                              int *err) {
     constexpr int U = 8;
-    for (int b0 = lane; b0 < nch; b0 += 32 * U) {
-        double t0[U], t1[U], t2[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int b = b0 + 32 * u;
-            const bool ok = b < nch;
-            t0[u] = ok ? __ldcg(chi + 3 * b) : 0.0;
-            t1[u] = ok ? __ldcg(chi + 3 * b + 1) : 0.0;
-            t2[u] = ok ? __ldcg(chi + 3 * b + 2) : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) { v0 += t0[u]; v1 += t1[u]; v2 = fmax(v2, t2[u]); }
-    }
+    const int lane = threadIdx.x & 31;
+    double v3 = 0.0, v4 = 0.0;
     for (int b0 = lane; b0 < nst; b0 += 32 * U) {
         double t3[U], t4[U];
 #pragma unroll
@@ -261,6 +243,35 @@ __device__ __forceinline__ void record_warp(const double *chi, int nch, const do
         if (write_ring) ring[step % M2M_HISTORY] = r;
         if (!(isfinite(v0) && isfinite(v3) && isfinite(v4))) atomicOr(err, ERR_NONFINITE);
     }
+}
+
+// The step record from the residual's per-block partials (chi^2, sum of
+// Delta^2, max |Delta~|: 3 doubles per block) and the pass's per-block
+// partials (S, sum w: 2 doubles per block), reduced by one warp in a fixed
+// order (lane k takes blocks k, k+32, ... in turn, then a fixed shuffle
+// tree): the same record whichever kernel computes it.  Lane 0 writes it.
+__device__ __forceinline__ void record_warp(const double *chi, int nch, const double *st, int nst, double mu,
+                                            long long step, int write_ring, m2m_record *ring, m2m_record *last,
+                                            int *err) {
+    const int lane = threadIdx.x & 31;
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+    // up to 8 partials per lane loaded before any is added (one memory
+    // latency instead of eight), then added in block order
+    constexpr int U = 8;
+    for (int b0 = lane; b0 < nch; b0 += 32 * U) {
+        double t0[U], t1[U], t2[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int b = b0 + 32 * u;
+            const bool ok = b < nch;
+            t0[u] = ok ? __ldcg(chi + 3 * b) : 0.0;
+            t1[u] = ok ? __ldcg(chi + 3 * b + 1) : 0.0;
+            t2[u] = ok ? __ldcg(chi + 3 * b + 2) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) { v0 += t0[u]; v1 += t1[u]; v2 = fmax(v2, t2[u]); }
+    }
+    record_finish(v0, v1, v2, st, nst, mu, step, write_ring, ring, last, err);
 }
 
 // ----------------------------------------------------------------- staging
@@ -1701,7 +1712,7 @@ void *pass_kernel_f32_steady(int layout, int pk = PK_ANY);
 void *pass_kernel_f32_compiled(int flags, int layout, int pk);   // NULL if not compiled
 void *pass_kernel_f32_pipe_steady(int layout);
 void *pass_kernel_f32_batch(int layout, bool steady = false, int pk = PK_ANY);
-void *steps_kernel_f32(int layout, int pk);                      // NULL if not compiled
+void *steps_kernel_f32(int layout, int pk, bool solo);                      // NULL if not compiled
 void *pass_kernel_f64(int threads, int layout);
 void *cells_kernel_f32();
 void *cells_kernel_f64();

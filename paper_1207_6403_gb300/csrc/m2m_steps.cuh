@@ -17,6 +17,18 @@
 //      Delta~ and the update's coefficients, and leaves its chi^2 partials;
 //   5. grid barrier; one warp writes the step record while the next
 //      step's particles run.
+// With at most SOLO_OBS observables (SOLO) every block forms the whole
+// residual by itself instead: steps 4 and 5 become the FP64 work of all
+// observables in one block (about 10 operations each, 1 us for 400) and save
+// a barrier and the coefficients' way through L2.  The totals then rotate
+// through three buffers: a block clears its slice of the next step's while
+// this step's particles run, when every block is past reading it (two steps
+// back).  Delta and Delta~ stay in shared memory and are written once, by
+// block 0, after the launch's last step.  Measured: 1M particles, 400
+// observables, 25 steps 765 us with the two barriers, 724 with one; a launch
+// of one or two steps gains nothing and takes the two.  (A kernel of its own:
+// both forms behind a run-time test made the layouts with thousands of
+// observables 4% slower.)
 // The arithmetic is that of k_pass and k_residual (the same particle and
 // residual functions), so the state after a launch equals, bit for bit,
 // the state after the same steps taken as one pass and one residual launch
@@ -40,10 +52,13 @@ struct StepsArgs {
     int last_range;               // the last step also takes the (E, L_z) range
     unsigned long long *bar;      // grid-barrier arrivals, zero at launch
     double *st2;                  // [2][grid][2]: S, sum w of each block, by step parity
+    unsigned long long *tot3;     // solo residual: [3][nobs] totals, zero at launch; else null
     double *chi2;                 // [2][grid][3]: chi^2, sum Delta^2, max |Delta~|, by step parity
     long long wait_ns;            // limit of one barrier wait (globaltimer ns)
     int test_stall;               // test only: block 0 never arrives at the first barrier
 };
+
+constexpr int SOLO_OBS = 512;
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -100,7 +115,8 @@ __device__ __forceinline__ void grid_barrier(unsigned long long *bar, unsigned l
 // The next chunk's state is loaded before the current one is processed.
 template <int L, int PK, int FL>
 __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSmem<float> &S, int G, int nit,
-                                                ThreadAcc &t, float fs, long long epoch, bool cache_read) {
+                                                ThreadAcc &t, float fs, long long epoch, bool cache_read,
+                                                unsigned long long *tot) {
     constexpr int NT = 1024;
     float *px = (float *)a.x, *py = (float *)a.y, *pz = (float *)a.z;
     float *pvx = (float *)a.vx, *pvy = (float *)a.vy, *pvz = (float *)a.vz;
@@ -151,7 +167,7 @@ __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSme
             // totals
             __syncthreads();
             fx_totals<L>(a, S, threadIdx.x >> 5, NT / 32, true, [&](int q, long long v) {
-                if (v) atomicAdd(a.y_acc + q, (unsigned long long)v);
+                if (v) atomicAdd(tot + q, (unsigned long long)v);
             });
             __syncthreads();
             it = 0;
@@ -159,9 +175,24 @@ __device__ __forceinline__ void steps_particles(const PassArgs &a, const PassSme
     }
 }
 
+// The record of a solo residual, by one warp: chi^2 from the observables'
+// Delta~ and Delta in shared memory.
+__device__ __forceinline__ void record_solo(const double *dt, const double *dd, int nobs, const double *st, int nst,
+                                            double mu, long long step, m2m_record *ring, m2m_record *last, int *err) {
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+    for (int j = threadIdx.x & 31; j < nobs; j += 32) {
+        const double a = dt[j], b = dd[j];
+        v0 = fma(a, a, v0);
+        v1 = fma(b, b, v1);
+        v2 = fmax(v2, fabs(a));
+    }
+    record_finish(v0, v1, v2, st, nst, mu, step, 1, ring, last, err);
+}
+
 // Dynamic shared memory: that of the steady pass of the same layout
-// (pass_smem_bytes with the steady flags).
-template <int L, int PK>
+// (pass_smem_bytes with the steady flags), and 16 bytes per observable for a
+// solo residual.
+template <int L, int PK, bool SOLO>
 __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ StepsArgs A) {
     constexpr int NT = 1024;
     using R = float;
@@ -186,6 +217,7 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
     S.ghc = (const float4 *)p; p += 48 * (a.gh_len / 5);
     if (L == 1) { S.pmap = (const short *)p; p += 2 * ((a.sets[1].pmap_len + 7) & ~7); }
     S.mmk = mmk;
+    double *sDt = (double *)p, *sD = sDt + nobs;         // solo: Delta~ and Delta
 
     const int G = (int)gridDim.x, b = (int)blockIdx.x;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -209,6 +241,8 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
     if (L == 1)
         for (int k = threadIdx.x; k < a.sets[1].pmap_len; k += NT) ((short *)S.pmap)[k] = a.sets[1].pmap[k];
     if (threadIdx.x == 0) { mmk[0] = fkey(INFINITY); mmk[1] = fkey(-INFINITY); mmk[2] = 0; }
+    if constexpr (SOLO)
+        for (int j = threadIdx.x; j < nobs; j += NT) sDt[j] = __ldcg(r.Dt + j);
 
     const float fs = a.fx_shift <= 127 ? __int_as_float((a.fx_shift + 127) << 23) : INFINITY;
     unsigned long long round = 0;
@@ -219,10 +253,16 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
         const bool cache_read = s > 0 || A.first_cache;
         const long long epoch = A.epoch0 + s;
         const int par = (int)((A.t0 + s) & 1);
+        unsigned long long *tot = SOLO ? A.tot3 + (size_t)(s % 3) * nobs : a.y_acc;
+        if (SOLO && s > 0) {
+            // (the first step's next buffer is clear already)
+            unsigned long long *nx = A.tot3 + (size_t)((s + 1) % 3) * nobs;
+            for (int j = j0 + (int)threadIdx.x; j < j1; j += NT) __stcg(nx + j, 0ull);
+        }
         // this step's coefficients (the previous step's residual wrote them
         // during this launch: read past L1); the histogram cleared while
         // they arrive
-        if (upd) {
+        if (upd && !(SOLO && s > 0)) {       // (a solo residual leaves them in shared memory)
             if (vec) {
                 for (int k = threadIdx.x; k < nobs / 4; k += NT)
                     ((float4 *)S.coef)[k] = __ldcg((const float4 *)r.coef_r + k);
@@ -256,16 +296,19 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
         // with the fewest particles) before its particles: its FP64 sums run
         // beside the other warps' particle work (the partials stay in place
         // until the next step's residual)
-        if (s > 0 && b == G - 1 && wp == NT / 32 - 1)
-            record_warp(A.chi2 + (size_t)3 * (par ^ 1) * G, G, A.st2 + (size_t)2 * (par ^ 1) * G, G, r.mu, A.t0 + s,
+        if (s > 0 && b == G - 1 && wp == NT / 32 - 1) {
+            if constexpr (SOLO)
+                record_solo(sDt, sD, nobs, A.st2 + (size_t)2 * (par ^ 1) * G, G, r.mu, A.t0 + s, r.ring, r.last, a.err);
+            else record_warp(A.chi2 + (size_t)3 * (par ^ 1) * G, G, A.st2 + (size_t)2 * (par ^ 1) * G, G, r.mu, A.t0 + s,
                         1, r.ring, r.last, a.err);
+        }
         ThreadAcc t{0.f, 0.f, false, false};
         if (upd) {
-            if (rng) steps_particles<L, PK, F_STEADY | F_MINMAX>(a, S, G, nit, t, fs, epoch, cache_read);
-            else steps_particles<L, PK, F_STEADY>(a, S, G, nit, t, fs, epoch, cache_read);
+            if (rng) steps_particles<L, PK, F_STEADY | F_MINMAX>(a, S, G, nit, t, fs, epoch, cache_read, tot);
+            else steps_particles<L, PK, F_STEADY>(a, S, G, nit, t, fs, epoch, cache_read, tot);
         } else {
-            if (rng) steps_particles<L, PK, F_PUSH | F_SCAT | F_STATS | F_MINMAX>(a, S, G, nit, t, fs, epoch, cache_read);
-            else steps_particles<L, PK, F_PUSH | F_SCAT | F_STATS>(a, S, G, nit, t, fs, epoch, cache_read);
+            if (rng) steps_particles<L, PK, F_PUSH | F_SCAT | F_STATS | F_MINMAX>(a, S, G, nit, t, fs, epoch, cache_read, tot);
+            else steps_particles<L, PK, F_PUSH | F_SCAT | F_STATS>(a, S, G, nit, t, fs, epoch, cache_read, tot);
         }
         ovf |= t.ovf;
         bad |= t.bad;
@@ -291,12 +334,34 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
             // totals (integer atomics: any order; a warp's 32 atomics on 32
             // consecutive totals, two cache lines)
             fx_totals<L>(a, S, wp - 1, NT / 32 - 1, false, [&](int k, long long v) {
-                if (v) atomicAdd(a.y_acc + k, (unsigned long long)v);
+                if (v) atomicAdd(tot + k, (unsigned long long)v);
             });
         }
         round += (unsigned long long)G;
         grid_barrier(A.bar, round, A.wait_ns, a.err, !(A.test_stall && b == 0 && s == 0));
 
+        if constexpr (SOLO) {
+            // all observables, by every block alike (one thread each)
+            const int j = (int)threadIdx.x;
+            if (j < nobs) {
+                const double yv = (double)(long long)__ldcg(tot + j) * r.q, is = __ldg(r.inv_sigma + j);
+                const bool valid = is > 0.0;
+                const double D = valid ? (yv - __ldg(r.Y + j)) * is : 0.0;
+                const double dn = r.alpha * D + (1.0 - r.alpha) * sDt[j];
+                const double cf = valid ? dn * is : 0.0;
+                sDt[j] = dn;
+                sD[j] = D;
+                ((R *)S.coef)[j] = (float)cf;
+                if (b == 0 && s == A.nsteps - 1) {
+                    r.y[j] = yv;
+                    r.Delta[j] = D;
+                    r.Dt[j] = dn;
+                    r.coef_d[j] = cf;
+                    ((float *)r.coef_r)[j] = (float)cf;
+                }
+            }
+            continue;
+        }
         // residual of the block's observables, one thread each: read and
         // clear their totals
         double c2 = 0.0, c2r = 0.0, mx = 0.0;
@@ -329,9 +394,12 @@ __global__ void __launch_bounds__(1024, 1) k_steps(const __grid_constant__ Steps
         grid_barrier(A.bar, round, A.wait_ns, a.err);
     }
     // the launch's last record
+    __syncthreads();
     if (b == G - 1 && wp == 0) {
         const int par = (int)((A.t0 + A.nsteps - 1) & 1);
-        record_warp(A.chi2 + (size_t)3 * par * G, G, A.st2 + (size_t)2 * par * G, G, r.mu, A.t0 + A.nsteps, 1,
+        if constexpr (SOLO)
+            record_solo(sDt, sD, nobs, A.st2 + (size_t)2 * par * G, G, r.mu, A.t0 + A.nsteps, r.ring, r.last, a.err);
+        else record_warp(A.chi2 + (size_t)3 * par * G, G, A.st2 + (size_t)2 * par * G, G, r.mu, A.t0 + A.nsteps, 1,
                     r.ring, r.last, a.err);
     }
     if (ovf) atomicOr(a.err, ERR_OVERFLOW);
