@@ -86,7 +86,11 @@ struct m2m_ctx {
     int rec_chi_nblk, rec_stat_par, rec_stat_nblk;
     unsigned long long *d_rec_ticket;
     unsigned long long rec_base;
-    m2m_record *d_ring, *d_last;
+    m2m_record *d_ring;
+    // what the m2m_get_* calls read, one block so that a call is one copy:
+    // [y | Delta | Delta~ | last record | error word]
+    double *d_out;
+    m2m_record *d_last;
     int *d_err;
     void *d_mm_slots;
     int mm_nblocks;
@@ -655,14 +659,18 @@ int finish_record(m2m_ctx *ctx) {
     return M2M_OK;
 }
 
-int check_err_word(m2m_ctx *ctx) {
-    int h = 0;
-    CU(cudaMemcpyAsync(&h, ctx->d_err, sizeof h, cudaMemcpyDeviceToHost, ctx->st));
-    CU(cudaStreamSynchronize(ctx->st));
+int err_word(m2m_ctx *ctx, int h) {
     if (h & ERR_NONFINITE) return set_err(ctx, M2M_ERR_NONFINITE, "a weight or a reduction became non-finite");
     if (h & ERR_OVERFLOW) return set_err(ctx, M2M_ERR_OVERFLOW, "fixed-point histogram range exceeded");
     if (h & ERR_TIMEOUT) return set_err(ctx, M2M_ERR_TIMEOUT, "a bounded device wait ran out (bulk copy or grid barrier; results invalid)");
     return M2M_OK;
+}
+
+int check_err_word(m2m_ctx *ctx) {
+    int h = 0;
+    CU(cudaMemcpyAsync(&h, ctx->d_err, sizeof h, cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaStreamSynchronize(ctx->st));
+    return err_word(ctx, h);
 }
 
 void free_events(m2m_ctx *c) {
@@ -674,9 +682,9 @@ void free_events(m2m_ctx *c) {
 
 void free_all(m2m_ctx *c) {
     free_events(c);
-    void *ptrs[] = {c->d_edges, c->d_gh, c->d_Y, c->d_sigma, c->d_isig, c->d_Dt, c->d_y, c->d_Delta, c->d_coef_d,
+    void *ptrs[] = {c->d_edges, c->d_gh, c->d_Y, c->d_sigma, c->d_isig, c->d_out, c->d_coef_d,
                     c->d_coef_r, c->d_slots, c->d_stat_slots, c->d_chi_slots, c->d_ticket, c->d_rec_ticket, c->d_ring,
-                    c->d_last, c->d_err, c->d_mm_slots, c->d_cell_ids, c->d_cell_acc, c->d_cell_cnt,
+                    c->d_mm_slots, c->d_cell_ids, c->d_cell_acc, c->d_cell_cnt,
                     c->d_cell_mean, c->d_cell_cache, c->d_y_acc, c->d_sh_e2, c->d_sh_rn, c->d_sh_irn,
                     c->d_sh_tab, c->d_sh_rnd, c->d_sh_sum, c->d_facc, c->d_lnwhat, c->d_lut, c->d_pmap, c->d_psf,
                     c->d_bar, c->d_st2, c->d_chi2, c->d_vm, c->d_c64, c->d_exp};
@@ -1032,9 +1040,15 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     size_t rs = f32 ? 4 : 8;
     ALLOC(ctx->d_edges, rs * ctx->edge_len);
     ALLOC(ctx->d_gh, rs * (ctx->gh_len + 1));
-    ALLOC(ctx->d_Y, 8 * nobs); ALLOC(ctx->d_sigma, 8 * nobs); ALLOC(ctx->d_Dt, 8 * nobs);
+    ALLOC(ctx->d_Y, 8 * nobs); ALLOC(ctx->d_sigma, 8 * nobs);
     ALLOC(ctx->d_isig, 8 * nobs);
-    ALLOC(ctx->d_y, 8 * nobs); ALLOC(ctx->d_Delta, 8 * nobs); ALLOC(ctx->d_coef_d, 8 * nobs);
+    ALLOC(ctx->d_coef_d, 8 * nobs);
+    ALLOC(ctx->d_out, 24 * (size_t)nobs + sizeof(m2m_record) + 8);
+    ctx->d_y = ctx->d_out;
+    ctx->d_Delta = ctx->d_y + nobs;
+    ctx->d_Dt = ctx->d_Delta + nobs;
+    ctx->d_last = (m2m_record *)(ctx->d_Dt + nobs);
+    ctx->d_err = (int *)(ctx->d_last + 1);
     ALLOC(ctx->d_coef_r, rs * nobs);
     if (f32) ALLOC(ctx->d_slots, (size_t)8 * nobs * ctx->slot_cap);
     if (!f32) ALLOC(ctx->d_exp, 8 * EXP_N);
@@ -1047,8 +1061,6 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     ALLOC(ctx->d_chi2, (size_t)48 * ctx->slot_cap);
     ALLOC(ctx->d_ticket, 4);
     ALLOC(ctx->d_ring, sizeof(m2m_record) * M2M_HISTORY);
-    ALLOC(ctx->d_last, sizeof(m2m_record));
-    ALLOC(ctx->d_err, 4);
     ALLOC(ctx->d_mm_slots, rs * 4 * ctx->slot_cap);
     ALLOC(ctx->d_cell_cache, 4 * (size_t)n);
     if (!lut_h.empty()) ALLOC(ctx->d_lut, 4 * lut_h.size());
@@ -1578,19 +1590,31 @@ int m2m_philox4x32_10(int64_t n, const uint32_t *counters, const uint32_t *keys,
 
 int m2m_get_obs(m2m_ctx *ctx, double *y, double *Delta, double *Dt) {
     if (!ctx) return M2M_ERR_ARG;
-    size_t b = 8 * (size_t)ctx->nobs;
-    if (y) CU(cudaMemcpyAsync(y, ctx->d_y, b, cudaMemcpyDeviceToHost, ctx->st));
-    if (Delta) CU(cudaMemcpyAsync(Delta, ctx->d_Delta, b, cudaMemcpyDeviceToHost, ctx->st));
-    if (Dt) CU(cudaMemcpyAsync(Dt, ctx->d_Dt, b, cudaMemcpyDeviceToHost, ctx->st));
-    return check_err_word(ctx);
+    if (!y && !Delta && !Dt) return check_err_word(ctx);
+    // one copy of the whole block: each pageable copy waits for the stream
+    // and costs the host about 8 us
+    const size_t b = 8 * (size_t)ctx->nobs, total = 3 * b + sizeof(m2m_record) + 4;
+    std::vector<unsigned char> h(total);
+    CU(cudaMemcpyAsync(h.data(), ctx->d_out, total, cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaStreamSynchronize(ctx->st));
+    if (y) memcpy(y, h.data(), b);
+    if (Delta) memcpy(Delta, h.data() + b, b);
+    if (Dt) memcpy(Dt, h.data() + 2 * b, b);
+    int e = 0;
+    memcpy(&e, h.data() + total - 4, 4);
+    return err_word(ctx, e);
 }
 
 int m2m_get_record(m2m_ctx *ctx, m2m_record *out) {
     if (!ctx || !out) return set_err(ctx, M2M_ERR_ARG, "NULL argument");
     int rc = finish_record(ctx);
     if (rc) return rc;
-    CU(cudaMemcpyAsync(out, ctx->d_last, sizeof *out, cudaMemcpyDeviceToHost, ctx->st));
-    return check_err_word(ctx);
+    struct { m2m_record r; int err; } h;       // as the block ends on the device
+    static_assert(sizeof(m2m_record) % 8 == 0, "the error word follows the record");
+    CU(cudaMemcpyAsync(&h, ctx->d_last, sizeof(m2m_record) + 4, cudaMemcpyDeviceToHost, ctx->st));
+    CU(cudaStreamSynchronize(ctx->st));
+    *out = h.r;
+    return err_word(ctx, h.err);
 }
 
 int m2m_get_record_async(m2m_ctx *ctx, m2m_record *out) {
@@ -2332,12 +2356,14 @@ int m2m_batch_get_records(m2m_batch *b, m2m_record *out) {
     unsigned char *g = (unsigned char *)b->d_gather;
     k_gather_records<<<(n + 127) / 128, 128, 0, b->st>>>((const m2m_record *const *)g, (const int *const *)(g + o_err),
                                                          n, (m2m_record *)(g + o_rec), (int *)(g + o_w));
-    std::vector<int> errw(n);
+    std::vector<unsigned char> h(bytes - o_rec);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, g + o_rec, sizeof(m2m_record) * n, cudaMemcpyDeviceToHost, b->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(errw.data(), g + o_w, 4 * (size_t)n, cudaMemcpyDeviceToHost, b->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h.data(), g + o_rec, h.size(), cudaMemcpyDeviceToHost, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "record gather: %s", cudaGetErrorString(e));
+    memcpy(out, h.data(), sizeof(m2m_record) * n);
+    std::vector<int> errw(n);
+    memcpy(errw.data(), h.data() + (o_w - o_rec), 4 * (size_t)n);
     for (int m = 0; m < n; ++m)
         if (errw[m]) return berr(b, check_err_word(b->ctx[m]), "model %d: %s", m, b->ctx[m]->err.c_str());
     return M2M_OK;
