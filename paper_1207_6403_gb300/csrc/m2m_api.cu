@@ -343,6 +343,13 @@ int detect_layout(const m2m_ctx *c) {
     return 0;
 }
 
+// The passes keep each particle's cells from the scatter for the update:
+// every compiled layout, and the FP32C run-time walk where the sets' cells fit
+// the packed word.
+bool keeps_cells(const m2m_ctx *c) {
+    return c->layout != 0 || (c->prec == M2M_FP32C && c->cache_bits <= 32);
+}
+
 LaunchShape pick_kernel(const m2m_ctx *c) {
     int nt = c->threads;
     // FP64, no shape asked for: 16 warps on an SM hide the FP64 latency better
@@ -398,8 +405,8 @@ void fill_args(const m2m_ctx *c, PassArgs &a, int flags) {
         }
     }
     a.cell_cache = c->d_cell_cache;
-    a.cache_read = (flags & F_UPD) && c->cache_valid && c->layout != 0;
-    a.cache_write = (flags & F_SCAT) && c->layout != 0;
+    a.cache_read = (flags & F_UPD) && c->cache_valid && keeps_cells(c);
+    a.cache_write = (flags & F_SCAT) && keeps_cells(c);
     a.cell_ids = c->d_cell_ids; a.cell_acc = c->d_cell_acc; a.cell_cnt = c->d_cell_cnt;
     a.err = c->d_err;
 }
@@ -470,7 +477,7 @@ int launch_pass(m2m_ctx *ctx, int flags, int *grid_out = nullptr) {
     if (flags & F_STATS) { ctx->stat_prev_nblk = (int)grid; ctx->stat_par ^= 1; }
     if (a.rec_pending) { ctx->rec_pending = false; ctx->rec_base += (unsigned long long)grid; }
     if (flags & F_MINMAX) ctx->mm_nblocks = (int)grid;
-    if (flags & F_SCAT) ctx->cache_valid = ctx->layout != 0;
+    if (flags & F_SCAT) ctx->cache_valid = keeps_cells(ctx);
     else if (flags & F_PUSH) ctx->cache_valid = false;
     if (flags & F_PUSH) ctx->facc_valid = ctx->sh_on && a.facc != nullptr;
     if (a.c64_lnw) {
@@ -956,6 +963,12 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
             edges_d.insert(edges_d.end(), e, e + nb + 1);
             if (ax == 0) { d.ex_off = off; guess_params(e, nb, &d.gx_mode, &d.gx_a, &d.gx_b); }
             else { d.ey_off = off; guess_params(e, nb, &d.gy_mode, &d.gy_a, &d.gy_b); }
+        }
+        if (s > 0 && o.geom == obs[s - 1].geom && o.geom != M2M_GEOM_LUT && !o.psf_q && !obs[s - 1].psf_q &&
+            d.nx == ctx->sets[s - 1].nx && d.ny == ctx->sets[s - 1].ny) {
+            const SetDev &e = ctx->sets[s - 1];
+            d.same = !memcmp(&edges_d[d.ex_off], &edges_d[e.ex_off], 8 * (size_t)(d.nx + 1)) &&
+                     (!two_d || !memcmp(&edges_d[d.ey_off], &edges_d[e.ey_off], 8 * (size_t)(d.ny + 1)));
         }
         if (o.quant == M2M_Q_GH) {
             if (!o.gh_V || !o.gh_S || !(o.sigma_kernel >= 0)) {

@@ -34,6 +34,7 @@ struct SetDev {
     int gx_mode, gy_mode; // index guess for the x / y edges
     float gx_a, gx_b, gy_a, gy_b;
     float gx_top, gy_top; // nx - 1, ny - 1 as floats (clamp of the guess)
+    int same;             // 1: geometry and edges of the set before it (its cell is the same)
     int cshift, cmask;    // packed cell cache: ((cell + 1) & cmask) << cshift
     const int *lut;       // geometry 4: device table of nx*ny cell ids (-1: none)
     const void *psf;      // seeing: 2^bits displacement quantiles (state precision), or null
@@ -928,7 +929,10 @@ __device__ __forceinline__ R potential(R x, R y, R z, const PassArgs &a, const R
 // (a.facc, [3][n] in the state precision) and, while neither the positions
 // nor the node table have changed since (a.facc_read), taken instead of a
 // second evaluation at the start of the next push: the same function of the
-// same arguments, so the same bits.
+// same arguments, so the same bits.  (FP64 keeps it for every potential inside
+// one m2m_step call.  FP32C potentials without an expansion do not: the 24
+// bytes cost more than a second evaluation, 10% of a step in the logarithmic
+// potential, 4% in Hernquist + NFW.)
 template <class R, int PK = PK_ANY>
 __device__ __forceinline__ void kdk(R &x, R &y, R &z, R &vx, R &vy, R &vz, const PassArgs &a,
                                     const R *sh = nullptr, long long i = 0) {
@@ -968,10 +972,11 @@ __device__ __forceinline__ int find_bin(R v, const R *e, int nb, int mode, float
     if (!(v >= e[0] && v < e[nb])) return -1;
     int j;
     if (mode == G_BIS) {
-        int lo = 0, hi = nb;              // e[lo] <= v < e[hi]
-        while (hi - lo > 1) {
-            int mid = (lo + hi) >> 1;
-            if (v >= e[mid]) lo = mid; else hi = mid;
+        // e[lo] <= v < e[nb]; the same steps for every lane, no branch
+        int lo = 0;
+        for (int step = 1 << (31 - __clz(nb)); step > 0; step >>= 1) {
+            const int mid = lo + step;
+            if (mid < nb && v >= e[mid]) lo = mid;
         }
         return lo;
     }

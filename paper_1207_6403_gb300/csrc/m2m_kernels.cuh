@@ -316,7 +316,7 @@ inline size_t pass_smem_bytes(bool f32, int layout, int flags, int nobs, int edg
     if (f32 || layout != 0) b += 2 * rs * (size_t)((edge_len + 1) & ~1);   // edge pairs (FP64: their keys)
     b += rs * (size_t)((gh_len + 3) & ~3);
     if (f32 && layout != 0) b += 48 * (size_t)(gh_len / 5);          // combined GH records
-    else if (!f32 && layout != 0 && (flags & F_UPD)) b += rs * (size_t)((gh_len + 3) & ~3);
+    else if ((flags & F_UPD) && (f32 || layout != 0)) b += rs * (size_t)((gh_len + 3) & ~3);   // the update's quartics
     if (f32 && layout == 1) b += 2 * (size_t)((pmap_len + 7) & ~7);   // pixel -> aperture table
     if (sh_len && (flags & (F_PUSH | F_MINMAX | F_CELLS))) b += rs * (size_t)((sh_len + 3) & ~3);
     if (flags & F_CELLS) {
@@ -343,6 +343,7 @@ struct PassSmem {
     int *hL, *hM, *hH;       // FP32C histogram: V = H * 2^32 + M * 2^16 + L per bin (exact fixed point)
     int hrep, hlane;         //   copies of L and M, and this lane's copy (see hist_copies)
     const R *coef, *edges, *gh;
+    const R *gpoly;          // run-time walk: the update's quartic of each GH cell, without the norm
     const Pair<R> *epair;    // (e[k], e[k+1]) for every edge-table index k
     const float4 *ghc;       // FP32C compiled layouts: per GH cell the three float4 of gh_record
     R *pe, *pl;
@@ -388,22 +389,31 @@ __device__ __forceinline__ R obs_dot(const PassArgs &a, const PassSmem<R> &S, R 
                                      long long i, long long epoch) {
     R dot = R(0);
     if constexpr (L == 0) {
+        int c = -1;
         for (int k = 0; k < a.nsets; ++k) {
             const SetDev &s = a.sets[k];
-            R Xk = X, Yk = Ys;
-            if (s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);
-            int c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
+            if (cached) {
+                c = (int)((cc >> s.cshift) & (unsigned)s.cmask) - 1;
+            } else if (!s.same) {
+                R Xk = X, Yk = Ys;
+                if (s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);
+                c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
+            }
             if (c < 0) continue;
-            int b = s.obs_off + c * s.nmom;
             if (s.quant == M2M_Q_MASS) {
-                dot = dot + S.coef[b];
+                dot = dot + S.coef[s.obs_off + c];
             } else if (s.quant == M2M_Q_VLOS2) {
-                dot = dot + (vlos * vlos) * S.coef[b];
+                dot = dot + (vlos * vlos) * S.coef[s.obs_off + c];
             } else {
-                R u[5];
-                gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
-#pragma unroll
-                for (int m = 0; m < 5; ++m) dot = dot + u[m] * S.coef[b + m];
+                // sum_n coef_n u_n(nu) = norm exp(-nu m / 2) P(m), m = nu c1
+                const R *g = S.gh + s.gh_off + 5 * c, *P = S.gpoly + s.gh_off + 5 * c;
+                const R nu = (vlos - g[0]) * g[1], m = nu * g[2];
+                const R e = g[4] * exp_ftz(-0.5f * nu * m);
+                R q = fmaf(P[4], m, P[3]);
+                q = fmaf(q, m, P[2]);
+                q = fmaf(q, m, P[1]);
+                q = fmaf(q, m, P[0]);
+                dot = dot + e * q;
             }
         }
     } else {
@@ -537,22 +547,33 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
     const int sh = a.fx_shift;
     unsigned packed = 0u;
     if constexpr (L == 0) {
+        int c = -1;
         for (int k = 0; k < a.nsets; ++k) {
             const SetDev &s = a.sets[k];
-            R Xk = X, Yk = Ys;
-            if (s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);
-            int c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
-            if (c < 0) continue;
-            const int b = s.obs_off + c * s.nmom, h = hist_at<L>(S, b, s.nmom);
-            if (s.quant == M2M_Q_MASS) {
-                hist_add(S, h, b, 0, wv, fs, sh, ovf);
-            } else if (s.quant == M2M_Q_VLOS2) {
-                hist_add(S, h, b, 0, wv * (vlos * vlos), fs, sh, ovf);
+            if (!s.same) {
+                R Xk = X, Yk = Ys;
+                if (s.psf) seeing<R>(s, k, i, epoch, Xk, Yk);
+                c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
+            }
+            packed |= (unsigned)(c + 1) << s.cshift;     // (kept only where the sets' fields fit)
+            if (c < 0 || wv == R(0)) continue;
+            const int b = s.obs_off + c * s.nmom;
+            if (s.quant != M2M_Q_GH) {
+                const R v = s.quant == M2M_Q_MASS ? wv : wv * (vlos * vlos);
+                const float Sv = v * fs;
+                if (fabsf(Sv) < FX_FAST) fx_red_fast(S.hL, S.hM, b, Sv);
+                else hist_add(S, b, b, 0, v, fs, sh, ovf);
             } else {
                 R u[5];
                 gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
+                // |u_n| <= sqrt 2 (below): one test for the five terms
+                if (fabsf(wv * fs) < 0.5f * FX_FAST) {
 #pragma unroll
-                for (int m = 0; m < 5; ++m) hist_add(S, h, b, m, wv * u[m], fs, sh, ovf);
+                    for (int m = 0; m < 5; ++m) fx_red_fast(S.hL, S.hM, b + m, (wv * u[m]) * fs);
+                } else {
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) hist_add(S, b, b, m, wv * u[m], fs, sh, ovf);
+                }
             }
         }
     } else {
@@ -672,7 +693,7 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
             const float wf = w_to_float(hi, lo);
             if (fl & F_UPD) {
                 const float vlos = vy * sn + vz * cs;
-                const bool cached = L != 0 && cache_read;
+                const bool cached = cache_read;
                 const float dot = obs_dot<R, L>(a, S, x, y, z, x, z * sn - y * cs, vlos, cached, cc, i, epoch);
                 const float Lw = lg2_ftz(wf) * LN2F - what;
                 const float G = a.f_mu * (-Lw - a.f_ent_c) - dot;
@@ -693,7 +714,7 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
             R wr;
             if (fl & F_UPD) {
                 R X = x, Ys = z * sn - y * cs, vlos = vy * sn + vz * cs;
-                const bool cached = L != 0 && cache_read;
+                const bool cached = cache_read;
                 R dot = obs_dot<R, L>(a, S, x, y, z, X, Ys, vlos, cached, cc, i, epoch);
                 wn = upd_weight(w, what, dot, a, wr, L1);
                 if (d_bad(wn)) t.bad = true;
@@ -722,7 +743,7 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
                                               epoch + ((fl & F_PUSH) ? 1 : 0));
         // (a pass with its flags compiled in always belongs to a context
         // with a cell cache; the run-time-flag passes ask)
-        if (L != 0 && (FL != 0 || a.cache_write)) a.cell_cache[i] = packed;
+        if ((L != 0 && FL != 0) || a.cache_write) a.cell_cache[i] = packed;
     }
     if (fl & F_MINMAX) {
         R E, Lz;
@@ -791,6 +812,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     S.gh = (const R *)p; p += sizeof(R) * ((a.gh_len + 3) & ~3);
     constexpr bool GHC = L != 0;      // combined GH records instead of gh + gpoly
     if (GHC) { S.ghc = (const float4 *)p; p += 48 * (a.gh_len / 5); }
+    else if (fl & F_UPD) { S.gpoly = (const R *)p; p += sizeof(R) * ((a.gh_len + 3) & ~3); }
     if (L == 1) { S.pmap = (const short *)p; p += 2 * ((a.sets[1].pmap_len + 7) & ~7); }
     const int sh_len = (a.sh_tab && (fl & (F_PUSH | F_MINMAX | F_CELLS))) ? a.sh_row * a.sh_K : 0;
     if (sh_len) { S.sh = (const R *)p; p += sizeof(R) * ((sh_len + 3) & ~3); }
@@ -831,6 +853,17 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     griddep_wait();
     if (fl & F_UPD) stage<4>((R *)S.coef, (const R *)a.coef, nobs, threadIdx.x, NT);
     if (sh_len) stage<4>((R *)S.sh, (const R *)a.sh_tab, sh_len, threadIdx.x, NT);
+    if (!GHC && (fl & F_UPD)) {
+        for (int k = 0; k < a.nsets; ++k) {
+            const SetDev &st = a.sets[k];
+            if (st.quant != M2M_Q_GH) continue;
+            for (int c = threadIdx.x; c < st.ncell; c += NT) {
+                const R *cf = (const R *)a.coef + st.obs_off + 5 * c;
+                gh_quartic<R>(((const R *)a.gh_tab)[st.gh_off + 5 * c + 3], R(1), cf[0], cf[1], cf[2], cf[3], cf[4],
+                              *(R (*)[5])(S.gpoly + st.gh_off + 5 * c));
+            }
+        }
+    }
     if constexpr (GHC) {
         // E[H_n] over N(m, t2) as polynomials in m (van der Marel & Franx
         // H_0..H_4), weighted by this step's coefficients of the cell (0
@@ -874,7 +907,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     const bool wr_w = (fl & F_UPD) != 0;
     const bool need_what = (fl & (F_UPD | F_STATS)) != 0;
     const R *pwh = (const R *)a.lnwhat;
-    const bool need_cc = L != 0 && a.cache_read && (fl & F_UPD);
+    const bool need_cc = a.cache_read && (fl & F_UPD);
     // FP32C histogram flush (all threads, after a barrier): the exact totals
     // H * 2^32 + M * 2^16 + L of this segment go into the global totals with
     // 64-bit integer atomics, or into this block's slot for the residual to
