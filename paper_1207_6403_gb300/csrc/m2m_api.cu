@@ -1270,14 +1270,23 @@ int m2m_get_sh_table(m2m_ctx *ctx, double *out) {
     if (!ctx || !out) return set_err(ctx, M2M_ERR_ARG, "NULL argument");
     if (!ctx->sh_on) return set_err(ctx, M2M_ERR_STATE, "the potential has no SH component");
     const size_t cnt = (size_t)ctx->sh_row * ctx->sh_K;
+    std::vector<double> v(cnt);
     if (ctx->prec == M2M_FP32C) {
         std::vector<float> f(cnt);
         CU(cudaMemcpyAsync(f.data(), ctx->d_sh_tab, 4 * cnt, cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));
-        for (size_t k = 0; k < cnt; ++k) out[k] = f[k];
+        for (size_t k = 0; k < cnt; ++k) v[k] = f[k];
     } else {
-        CU(cudaMemcpyAsync(out, ctx->d_sh_tab, 8 * cnt, cudaMemcpyDeviceToHost, ctx->st));
+        CU(cudaMemcpyAsync(v.data(), ctx->d_sh_tab, 8 * cnt, cudaMemcpyDeviceToHost, ctx->st));
         CU(cudaStreamSynchronize(ctx->st));
+    }
+    // the kernels' quadruples per term, then the radii, to the rows described
+    const size_t K = ctx->sh_K, row = ctx->sh_row, nt = (row - 1) / 4;
+    for (size_t k = 0; k < K; ++k) {
+        for (size_t t = 0; t < nt; ++t) {
+            for (size_t q = 0; q < 4; ++q) out[k * row + q * nt + t] = v[(k * nt + t) * 4 + q];
+        }
+        out[k * row + 4 * nt] = v[K * 4 * nt + k];
     }
     return M2M_OK;
 }

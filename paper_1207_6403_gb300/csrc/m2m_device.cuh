@@ -55,14 +55,13 @@ struct PotDev {
     float cf[6];          // the same rounded once to float (no per-particle conversions)
 };
 
-// Spherical-harmonic node table: one row of SH_ROW values per radial node k
-// (0..K-1), in the state precision:
-//   [0..4]   F_l(r_k)          l = 0, 2, 4, 6, 8
-//   [5..9]   dF_l per unit r to node k+1 (slope of the linear interpolant)
-//   [10..14] D_l(r_k)  (= dF_l/dr at the node)
-//   [15..19] slope of D_l to node k+1
-//   [20]     r_k
-// The last row has zero slopes.
+// Node table of an expansion of NT terms (5 for the axisymmetric one) with K
+// radial nodes, in the state precision: per node k and term t the quadruple
+//   F_t(r_k), its slope to node k+1 (of the linear interpolant),
+//   D_t(r_k) (= dF_t/dr at the node), its slope
+// (zero slopes at the last node), K rows of 4 NT values, then the K radii r_k:
+// a term is one 16-byte load, and rows of 20, 60 or 100 floats start on 8
+// different groups of banks.  SH_ROW etc.: values per node.
 constexpr int SH_ROW = 21;
 constexpr int SH_MAXK = 512;
 
@@ -389,6 +388,28 @@ __device__ __forceinline__ void legendre_even(R mu, R P[5], R dP[5]) {
     dP[4] = dP[3] + R(15) * p7;
 }
 
+// One term of a node: F, its slope, D, its slope.
+template <class R> struct NodeTerm { R f, fs, d, ds; };
+__device__ __forceinline__ NodeTerm<float> node_term(const float *q) {
+    const float4 v = *(const float4 *)q;
+    return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ NodeTerm<double> node_term(const double *q) {
+    const double2 a = *(const double2 *)q, b = *(const double2 *)(q + 2);
+    return {a.x, a.y, b.x, b.y};
+}
+
+// The segment [r_k, r_(k+1)) that holds r (r_0 <= r < r_(K-1)): a guess from
+// log2 r, then fixed by the node radii.
+template <class R>
+__device__ __forceinline__ int node_segment(R r, const R *rad, const PotDev &p) {
+    const float lg = fmaf(__log2f((float)r), p.cf[3], p.cf[4]) - 0.5f;
+    int k = rint_small(fminf(fmaxf(lg, 0.0f), (float)(p.ik - 2)));
+    while (k > 0 && r < rad[k]) --k;
+    while (k < p.ik - 2 && r >= rad[k + 1]) ++k;
+    return k;
+}
+
 // F_l(r), D_l(r) from the node table: linear between nodes, the exterior law
 // F_l(K-1) (r_(K-1)/r)^(l+1) beyond the last node, and inside the first
 // F_l(0) (r/r_0)^l, D_l(0) (r/r_0)^max(l-1, 1).
@@ -397,39 +418,36 @@ __device__ __forceinline__ void sh_radial(R r, R ir, const R *T, const PotDev &p
     const int K = p.ik;
     const R r0 = KC(R, p.c[1], p.cf[1]), rK = KC(R, p.c[2], p.cf[2]);
     if (r >= rK) {
-        const R *row = T + (K - 1) * SH_ROW;
+        const R *row = T + (K - 1) * 20;
         const R q = rK * ir, q2 = q * q;
         R qq = q;
 #pragma unroll
         for (int n = 0; n < 5; ++n) {
-            F[n] = row[n] * qq;
+            F[n] = row[4 * n] * qq;
             D[n] = -(R(2 * n + 1) * F[n]) * ir;
             qq = qq * q2;
         }
     } else if (r < r0) {
         const R q = r * KC(R, p.c[5], p.cf[5]), q2 = q * q;
         F[0] = T[0];
-        D[0] = T[10] * q;
+        D[0] = T[2] * q;
         R ql = q2, qd = q;
 #pragma unroll
         for (int n = 1; n < 5; ++n) {
-            F[n] = T[n] * ql;
-            D[n] = T[10 + n] * qd;
+            F[n] = T[4 * n] * ql;
+            D[n] = T[4 * n + 2] * qd;
             ql = ql * q2;
             qd = qd * q2;
         }
     } else {
-        // segment guess from log2 r, then fixed by the node radii
-        const float lg = fmaf(__log2f((float)r), p.cf[3], p.cf[4]) - 0.5f;
-        int k = rint_small(fminf(fmaxf(lg, 0.0f), (float)(K - 2)));
-        while (k > 0 && r < T[k * SH_ROW + 20]) --k;
-        while (k < K - 2 && r >= T[(k + 1) * SH_ROW + 20]) ++k;
-        const R *row = T + k * SH_ROW;
-        const R dr = r - row[20];
+        const R *rad = T + 20 * K;
+        const int k = node_segment<R>(r, rad, p);
+        const R dr = r - rad[k];
 #pragma unroll
         for (int n = 0; n < 5; ++n) {
-            F[n] = row[n] + dr * row[5 + n];
-            D[n] = row[10 + n] + dr * row[15 + n];
+            const NodeTerm<R> q = node_term(T + 20 * k + 4 * n);
+            F[n] = q.f + dr * q.fs;
+            D[n] = q.d + dr * q.ds;
         }
     }
 }
@@ -572,25 +590,23 @@ __device__ __forceinline__ void ex_terms(R mu, R nx, R ny, Fn &&f) {
     }
 }
 
-// Radial factors of a point: F_t(r) = T[t] fa_slot + dr T[NT+t] and
-// D_t(r) = T[2NT+t] da_slot + dr T[3NT+t] + (l+1) dbs F_t(r) from one table
-// row: linear between nodes (fa = da = 1, dbs = 0); beyond the last node
-// F(K-1) (r_(K-1)/r)^(l+1) and D = -(l+1) F/r (dr = 0, da = 0, dbs = -1/r);
-// inside the first F(0) (r/r_0)^l and D(0) (r/r_0)^max(l-1, 1) (dr = 0).
+// Radial factors of a point outside the nodes' range, from one table row
+// (quadruples q of the term): F_t = q.f fa_slot and D_t = q.d da_slot +
+// (l+1) dbs F_t; beyond the last node F(K-1) (r_(K-1)/r)^(l+1) and D =
+// -(l+1) F/r (da = 0, dbs = -1/r); inside the first F(0) (r/r_0)^l and D(0)
+// (r/r_0)^max(l-1, 1) (dbs = 0).
 template <class R> struct ExRad {
     const R *row;
-    R dr, dbs, fa[5], da[5];
+    R dbs, fa[5], da[5];
 };
 
 template <class B, class R>
 __device__ __forceinline__ void ex_rad(R r, R ir, const R *T, const PotDev &p, ExRad<R> &g) {
-    constexpr int NT = B::NT, ROW = B::ROW, S = B::LSTEP;
-    const int K = p.ik;
-    const R r0 = KC(R, p.c[1], p.cf[1]), rK = KC(R, p.c[2], p.cf[2]);
+    constexpr int S = B::LSTEP;
+    const R rK = KC(R, p.c[2], p.cf[2]);
     g.dbs = R(0);
-    g.dr = R(0);
     if (r >= rK) {
-        g.row = T + (K - 1) * ROW;
+        g.row = T + (p.ik - 1) * 4 * B::NT;
         const R q = rK * ir, qs = S == 2 ? q * q : q;
         g.fa[0] = q;
 #pragma unroll
@@ -598,7 +614,7 @@ __device__ __forceinline__ void ex_rad(R r, R ir, const R *T, const PotDev &p, E
 #pragma unroll
         for (int n = 0; n < 5; ++n) g.da[n] = R(0);
         g.dbs = -ir;
-    } else if (r < r0) {
+    } else {
         g.row = T;
         const R q = r * KC(R, p.c[5], p.cf[5]), qs = S == 2 ? q * q : q;
         g.fa[0] = R(1);
@@ -611,21 +627,32 @@ __device__ __forceinline__ void ex_rad(R r, R ir, const R *T, const PotDev &p, E
             const int l = n * S;
             g.da[n] = l <= 2 ? q : g.da[n - 1] * qs;
         }
-    } else {
-        const float lg = fmaf(__log2f((float)r), p.cf[3], p.cf[4]) - 0.5f;
-        int k = rint_small(fminf(fmaxf(lg, 0.0f), (float)(K - 2)));
-        while (k > 0 && r < T[k * ROW + 4 * NT]) --k;
-        while (k < K - 2 && r >= T[(k + 1) * ROW + 4 * NT]) ++k;
-        g.row = T + k * ROW;
-        g.dr = r - g.row[4 * NT];
-#pragma unroll
-        for (int n = 0; n < 5; ++n) { g.fa[n] = R(1); g.da[n] = R(1); }
     }
 }
 
-template <class B, class R>
-__device__ __forceinline__ R ex_F(const ExRad<R> &g, int t, int l) {
-    return g.row[t] * g.fa[B::slot(l)] + g.dr * g.row[B::NT + t];
+// Calls f(t, l, m, c, q0, q1, C, gx, gy, F_t(r), D_t(r)) for every term (see
+// ex_terms): linear between the nodes, where nearly every particle is, with
+// nothing but two multiply-adds per term; the factors of ex_rad elsewhere.
+template <class B, class R, class Fn>
+__device__ __forceinline__ void ex_radial_terms(R r, R ir, R mu, R nx, R ny, const R *T, const PotDev &p, Fn &&f) {
+    const R r0 = KC(R, p.c[1], p.cf[1]), rK = KC(R, p.c[2], p.cf[2]);
+    if (r >= r0 && r < rK) {
+        const R *rad = T + 4 * B::NT * p.ik;
+        const int k = node_segment<R>(r, rad, p);
+        const R dr = r - rad[k], *row = T + 4 * B::NT * k;
+        ex_terms<B, R>(mu, nx, ny, [&](int t, int l, int m, R c, R q0, R q1, R C, R gx, R gy) {
+            const NodeTerm<R> q = node_term(row + 4 * t);
+            f(t, l, m, c, q0, q1, C, gx, gy, q.f + dr * q.fs, q.d + dr * q.ds);
+        });
+    } else {
+        ExRad<R> g;
+        ex_rad<B, R>(r, ir, T, p, g);
+        ex_terms<B, R>(mu, nx, ny, [&](int t, int l, int m, R c, R q0, R q1, R C, R gx, R gy) {
+            const R F = g.row[4 * t] * g.fa[B::slot(l)];
+            f(t, l, m, c, q0, q1, C, gx, gy, F,
+              g.row[4 * t + 2] * g.da[B::slot(l)] + R(l + 1) * g.dbs * F);
+        });
+    }
 }
 
 template <class B, class R>
@@ -634,17 +661,26 @@ __device__ __forceinline__ void ex_accel(R x, R y, R z, const R *T, const PotDev
     if (!(r2 > R(0))) return;
     const R r = sqrt(r2), ir = R(1) / r;
     const R nx = x * ir, ny = y * ir, mu = z * ir;
-    ExRad<R> rd;
-    ex_rad<B, R>(r, ir, T, p, rd);
     R ar = R(0), az = R(0), ax = R(0), ay = R(0);   // along n, e_z, and G (the last two / r)
-    ex_terms<B, R>(mu, nx, ny, [&](int t, int l, int m, R c, R q0, R q1, R C, R gx, R gy) {
-        const R F = ex_F<B, R>(rd, t, l);
-        const R D = rd.row[2 * B::NT + t] * rd.da[B::slot(l)] + rd.dr * rd.row[3 * B::NT + t] +
-                    R(l + 1) * rd.dbs * F;
+    ex_radial_terms<B, R>(r, ir, mu, nx, ny, T, p,
+                          [&](int, int l, int m, R c, R q0, R q1, R C, R gx, R gy, R F, R D) {
         const R cq0C = c * q0 * C, Fc = F * c;
-        // D Y n + F c [q1 C (e_z - mu n) - m q0 C n + m q0 G] / r
-        ar = ar + (D * cq0C - (Fc * q1 * C * mu + F * R(m) * cq0C) * ir);
-        az = az + Fc * q1 * C;
+        // D Y n + F c [q1 C (e_z - mu n) - m q0 C n + m q0 G] / r, without the
+        // parts that are zero (q1 at l = m, the last two at m = 0; l and m
+        // are constants of the unrolled terms)
+        if (l == m && m == 0) {
+            ar = ar + D * cq0C;
+        } else if (l == m) {
+            ar = ar + (D * cq0C - (F * R(m) * cq0C) * ir);
+        } else if (m == 0) {
+            const R q1C = Fc * q1 * C;
+            ar = ar + (D * cq0C - (q1C * mu) * ir);
+            az = az + q1C;
+        } else {
+            const R q1C = Fc * q1 * C;
+            ar = ar + (D * cq0C - (q1C * mu + F * R(m) * cq0C) * ir);
+            az = az + q1C;
+        }
         if (m > 0) {
             const R s = Fc * R(m) * q0;
             ax = ax + s * gx;
@@ -662,12 +698,9 @@ __device__ __forceinline__ R ex_phi(R x, R y, R z, const R *T, const PotDev &p) 
     const R r = sqrt(r2);
     const R ir = r2 > R(0) ? R(1) / r : R(0);
     const R nx = x * ir, ny = y * ir, mu = r2 > R(0) ? z * ir : R(1);
-    ExRad<R> rd;
-    ex_rad<B, R>(r, ir, T, p, rd);
     R s = R(0);
-    ex_terms<B, R>(mu, nx, ny, [&](int t, int l, int m, R c, R q0, R q1, R C, R gx, R gy) {
-        s = s + c * q0 * C * ex_F<B, R>(rd, t, l);
-    });
+    ex_radial_terms<B, R>(r, ir, mu, nx, ny, T, p,
+                          [&](int, int, int, R c, R q0, R, R C, R, R, R F, R) { s = s + c * q0 * C * F; });
     return -s;
 }
 

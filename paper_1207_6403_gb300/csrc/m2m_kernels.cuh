@@ -1560,14 +1560,14 @@ __global__ void __launch_bounds__(256) k_sh_tables(const long long *sum, int K, 
     }
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        R *row = tab + (size_t)k * SH_ROW;
+        R *q = tab + ((size_t)k * 5 + n) * 4;
         const bool last = k == K - 1;
         const double h = last ? 1.0 : 1.0 / (rn[k + 1] - rn[k]);
-        row[n] = (R)F[k];
-        row[10 + n] = (R)D[k];
-        row[5 + n] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
-        row[15 + n] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
-        if (n == 0) row[20] = (R)rn[k];
+        q[0] = (R)F[k];
+        q[1] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
+        q[2] = (R)D[k];
+        q[3] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
+        if (n == 0) tab[(size_t)K * 20 + k] = (R)rn[k];
     }
 }
 
@@ -1682,7 +1682,7 @@ template <class B, class R>
 __global__ void __launch_bounds__(256) k_ex_tables(const long long *sum, int K, const double *rn, double q, R *tab,
                                                    int *err) {
     extern __shared__ __align__(16) double sd[];
-    constexpr int NT = B::NT, ROW = B::ROW;
+    constexpr int NT = B::NT;
     const int t = blockIdx.x, l = B::l_of(t);
     double *F = sd + 2 * K, *D = sd + 3 * K;
     node_sums<R>(sum, t, NT + t, l, K, rn, q, sd);
@@ -1699,14 +1699,14 @@ __global__ void __launch_bounds__(256) k_ex_tables(const long long *sum, int K, 
     }
     __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
-        R *row = tab + (size_t)k * ROW;
+        R *q = tab + ((size_t)k * NT + t) * 4;
         const bool last = k == K - 1;
         const double h = last ? 1.0 : 1.0 / (rn[k + 1] - rn[k]);
-        row[t] = (R)F[k];
-        row[2 * NT + t] = (R)D[k];
-        row[NT + t] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
-        row[3 * NT + t] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
-        if (t == 0) row[4 * NT] = (R)rn[k];
+        q[0] = (R)F[k];
+        q[1] = last ? R(0) : (R)((F[k + 1] - F[k]) * h);
+        q[2] = (R)D[k];
+        q[3] = last ? R(0) : (R)((D[k + 1] - D[k]) * h);
+        if (t == 0) tab[(size_t)K * 4 * NT + k] = (R)rn[k];
     }
 }
 
