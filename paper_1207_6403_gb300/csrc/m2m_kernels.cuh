@@ -683,6 +683,8 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
     const int fl = FL ? FL : a.flags;
     const R sn = KC(R, a.sin_i, a.f_sin_i), cs = KC(R, a.cos_i, a.f_cos_i);
     double wn = w;
+    Acc3<R> g0{R(0), R(0), R(0)};
+    if (fl & F_PUSH) g0 = kept_force<R, PK>(a, i);
     // a weight in the normal float range: the float arithmetic of
     // the update and the entropy on the two words of the double directly
     bool fast = false;
@@ -727,7 +729,7 @@ __device__ __forceinline__ void particle(const PassArgs &a, const PassSmem<R> &S
             t.bad = true;       // negative, -0 or NaN weight
         }
     }
-    if (fl & F_PUSH) kdk<R, PK>(x, y, z, vx, vy, vz, a, S.sh, i);
+    if (fl & F_PUSH) kdk<R, PK>(x, y, z, vx, vy, vz, a, S.sh, i, g0);
     if (fl & F_SCAT) {
         R X = x, Ys = z * sn - y * cs, vlos = vy * sn + vz * cs;
         // the scattered weight is a function of the stored (double) weight

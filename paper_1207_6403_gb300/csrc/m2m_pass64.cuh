@@ -295,7 +295,7 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
                 bad = true;       // negative, -0 or NaN weight
             }
         }
-        if (fl & F_PUSH) kdk<double, PK_ANY>(x, y, z, vx, vy, vz, a, sh, i);
+        if (fl & F_PUSH) kdk<double, PK_ANY>(x, y, z, vx, vy, vz, a, sh, i, kept_force<double, PK_ANY>(a, i));
         if (fl & F_SCAT) {
             const double X = x, Ys = z * sn - y * cs, vlos = vy * sn + vz * cs;
             if constexpr (L == 0) {
