@@ -1168,8 +1168,8 @@ __device__ __forceinline__ int find_fast(R v, const Pair<R> *e, int nb, float ga
     const float gf = fminf(fmaxf(fmaf(ga, t, gb) - 0.5f, 0.0f), top);
     int g = rint_small(gf);
     const Pair<R> ed = e[g];
-    g += (v >= ed.y ? 1 : 0) - (v < ed.x ? 1 : 0);
-    return ((unsigned)g < (unsigned)nb && v == v) ? g : -1;
+    g += (v >= ed.y ? 1 : 0) - (v >= ed.x ? 0 : 1);          // (NaN: guess 0, so -1)
+    return (unsigned)g < (unsigned)nb ? g : -1;
 }
 
 // Cell of a particle in a set of compile-time geometry G whose edge tables
@@ -1193,18 +1193,25 @@ __device__ __forceinline__ int cell_t(const SetDev &s, const Pair<R> *edges, R x
 }
 
 // Fixed-point histogram add of a float term v, V = round(v * 2^sh) (a
-// 64-bit integer), kept as three int32 sums per bin in shared memory:
-// V = A * 2^32 + B * 2^16 + L with |B| <= 2^15 and |L| <= 2^16.  Every part
-// goes in with a plain reduction (no returned value, no carry), and the bin
-// total is A_sum * 2^32 + B_sum * 2^16 + L_sum.  It is exact while at most
-// 2^15 terms reach a bin between two flushes (the pass flushes every
-// 32768 particles of a block), which keeps |B_sum|, |L_sum| < 2^31; A_sum
-// stays in range for any |V| < 2^62.  A is 0 for the usual terms (|V| <
-// 2^31, the fast path: V by one round-to-nearest conversion, L = V mod 2^16
-// and B = V >> 16) and its reduction is skipped.  For |V| < 2^38 the split
+// 64-bit integer), V = A * 2^32 + B * 2^16 + l with |B| <= 2^15 and l in
+// [-2^15, 2^16), kept as three int32 sums per bin in shared memory: A, B and
+// V mod 2^32 (wrapping; cheaper to add than l alone, one operation per term).
+// Every part goes in with a plain reduction (no returned value, no carry).
+// The sum of the l is (V_sum - B_sum * 2^16) mod 2^32 as a signed number, and
+// the bin total A_sum * 2^32 + B_sum * 2^16 + l_sum (see fx_total).  It is
+// exact while at most 2^15 terms reach a bin between two flushes (the pass
+// flushes every 32768 particles of a block), which keeps |B_sum| < 2^31 and
+// l_sum in [-2^30, 2^31); A_sum stays in range for any |V| < 2^62.  A is 0
+// for the usual terms (|V| < 2^31, the fast path: V by one round-to-nearest
+// conversion, B = V >> 16) and its reduction is skipped.  For |V| < 2^38 the split
 // takes two exact float steps (1.5*2^23 "magic" rounding of V/2^16, then of
 // the exact remainder V - h*2^16), larger terms take the bit-level path.
 // fscale = 2^sh as a float (an exact power of two).
+__device__ __forceinline__ long long fx_total(int vsum, int bsum, int asum) {
+    const int l = (int)((unsigned)vsum - ((unsigned)bsum << 16));
+    return (long long)(((unsigned long long)(long long)asum << 32) + ((unsigned long long)(long long)bsum << 16) +
+                       (unsigned long long)(long long)l);
+}
 constexpr float FX_MAGIC = 12582912.0f;            // 1.5 * 2^23
 // The common case of fx_red, for |S| = |v * 2^sh| < 2^31 (A = 0): the two
 // lower parts only, no range test; the caller checks the range once for all
@@ -1212,7 +1219,7 @@ constexpr float FX_MAGIC = 12582912.0f;            // 1.5 * 2^23
 constexpr float FX_FAST = 2147483648.0f;           // 2^31
 __device__ __forceinline__ void fx_red_fast(int *Lo, int *Mid, int b, float S) {
     const int V = __float2int_rn(S);                           // round to nearest even, |S| < 2^31
-    atomicAdd(Lo + b, V & 0xFFFF);
+    atomicAdd(Lo + b, V);
     atomicAdd(Mid + b, V >> 16);
 }
 // The five Gauss-Hermite terms of one particle (the arithmetic of
@@ -1243,15 +1250,17 @@ __device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, int hb
         const float r = fmaf(-(t - FX_MAGIC), 65536.0f, S);    // S - h * 2^16, exact
         l = __float_as_int(r + FX_MAGIC) - 0x4B400000;
         const int A = (h + 32768) >> 16;
-        atomicAdd(Lo + b, l);
-        atomicAdd(Mid + b, h - (A << 16));
+        const int mid = h - (A << 16);
+        atomicAdd(Lo + b, l + (int)((unsigned)mid << 16));
+        atomicAdd(Mid + b, mid);
         if (A) atomicAdd(Hi + hb, A);
     } else {
         const long long q = f2fixed(v, sh, ovf);
         const long long hh = (q + 32768) >> 16;
         const long long A = (hh + 32768) >> 16;
-        atomicAdd(Lo + b, (int)(q - (hh << 16)));
-        atomicAdd(Mid + b, (int)(hh - (A << 16)));
+        const int mid = (int)(hh - (A << 16));
+        atomicAdd(Lo + b, (int)(q - (hh << 16)) + (int)((unsigned)mid << 16));
+        atomicAdd(Mid + b, mid);
         atomicAdd(Hi + hb, (int)A);
     }
 }

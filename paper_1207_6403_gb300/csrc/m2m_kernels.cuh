@@ -340,7 +340,7 @@ template <int L> constexpr bool hist_copied = L == 2 || L == 3;
 
 template <class R>
 struct PassSmem {
-    int *hL, *hM, *hH;       // FP32C histogram: V = H * 2^32 + M * 2^16 + L per bin (exact fixed point)
+    int *hL, *hM, *hH;       // FP32C histogram: sums of V mod 2^32, B and A per bin (exact, see fx_red)
     int hrep, hlane;         //   copies of L and M, and this lane's copy (see hist_copies)
     const R *coef, *edges, *gh;
     const R *gpoly;          // run-time walk: the update's quartic of each GH cell, without the norm
@@ -490,7 +490,7 @@ __device__ __forceinline__ void hist_add(const PassSmem<float> &S, int i, int b,
                                          ThreadAcc &t) {
     fx_red(S.hL, S.hM, S.hH, i + m, b + m, v, fs, sh, t.ovf);
 }
-// The exact totals H * 2^32 + M * 2^16 + L of the block's FP32C histogram,
+// The exact totals (fx_total) of the block's FP32C histogram,
 // f(j, total) for every observable j, by `nw` warps of which this is `w`
 // (whole warps, after a barrier); clear: the histogram is zeroed for the next
 // segment.  With copies, two lanes share an observable, each summing half of
@@ -500,10 +500,7 @@ template <int L, class F>
 __device__ __forceinline__ void fx_totals(const PassArgs &a, const PassSmem<float> &S, int w, int nw, bool clear,
                                           F &&f) {
     const int lane = threadIdx.x & 31, nobs = a.nobs;
-    auto total = [&](int k, int lo, int mid) {
-        return (long long)(((unsigned long long)(long long)S.hH[k] << 32) +
-                           ((unsigned long long)(long long)mid << 16) + (unsigned long long)(long long)lo);
-    };
+    auto total = [&](int k, int lo, int mid) { return fx_total(lo, mid, S.hH[k]); };
     if (!hist_copied<L> || S.hrep == 1) {
         for (int k = 32 * w + lane; k < nobs; k += 32 * nw) {
             const long long v = total(k, S.hL[k], S.hM[k]);
@@ -911,7 +908,7 @@ __device__ __forceinline__ void pass_body(const PassArgs &a, const int bid, cons
     const R *pwh = (const R *)a.lnwhat;
     const bool need_cc = a.cache_read && (fl & F_UPD);
     // FP32C histogram flush (all threads, after a barrier): the exact totals
-    // H * 2^32 + M * 2^16 + L of this segment go into the global totals with
+    // (fx_total) of this segment go into the global totals with
     // 64-bit integer atomics, or into this block's slot for the residual to
     // sum (integer sums: the result does not depend on the order).
     int nseg = 0;
