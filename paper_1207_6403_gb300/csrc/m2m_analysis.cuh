@@ -16,6 +16,13 @@ __device__ __forceinline__ double rcp_d(double d) {
     return fma(y, fma(e, e, e), y);
 }
 
+// Float -> double exactly, with integer instructions for normal numbers (the
+// conversion instruction runs on the FP64 pipe).
+__device__ __forceinline__ double widen(float f) {
+    return (__float_as_uint(f) & 0x7f800000u) - 1u < 0x7f7fffffu ? f2d_fast(f) : (double)f;
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
 // Lane copies of the block's sums: lane l of every warp adds to copy
 // l mod copies, so that the lanes of a warp, which mostly share a shell, do
 // not queue on one address (a double shared-memory add is a compare-and-swap
@@ -38,7 +45,7 @@ inline int vmoments_copies(int nsh) {
 template <class R>
 __global__ void __launch_bounds__(256) k_vmoments(const R *x, const R *y, const R *z, const R *vx, const R *vy,
                                                   const R *vz, const double *w, long long n, const R *e2,
-                                                  int nsh, int copies, double *out) {
+                                                  int nsh, int copies, double *out, const int *err) {
     extern __shared__ __align__(16) unsigned char smem[];
     double *acc = (double *)smem;                           // [4 nsh][copies]
     R *ed = (R *)(acc + (size_t)4 * nsh * copies);
@@ -47,6 +54,8 @@ __global__ void __launch_bounds__(256) k_vmoments(const R *x, const R *y, const 
     __syncthreads();
     double *mine = acc + (threadIdx.x & (copies - 1));
     const R e_lo = ed[0], e_hi = ed[nsh];
+    // the context's error word after the sums, so that the caller reads both at once
+    if (blockIdx.x == 0 && threadIdx.x == 0) *(int *)(out + 4 * nsh) = *err;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const R xs = x[i], ys = y[i], zs = z[i], us = vx[i], vs = vy[i], ws = vz[i];
         const double wi = w[i];
@@ -57,7 +66,7 @@ __global__ void __launch_bounds__(256) k_vmoments(const R *x, const R *y, const 
             const int mid = (lo + hi) >> 1;
             if (ed[mid] <= q2) lo = mid; else hi = mid;
         }
-        const double X = xs, Y = ys, Z = zs, U = us, V = vs, W = ws;
+        const double X = widen(xs), Y = widen(ys), Z = widen(zs), U = widen(us), V = widen(vs), W = widen(ws);
         const double R2 = fma(X, X, Y * Y), r2 = fma(Z, Z, R2);
         const double s = fma(X, U, fma(Y, V, Z * W)), t = fma(X, V, -(Y * U));
         const double v2 = fma(U, U, fma(V, V, W * W));

@@ -1416,11 +1416,11 @@ int m2m_velocity_moments(m2m_ctx *ctx, const double *r2_edges, int32_t nshell, d
             return set_err(ctx, M2M_ERR_ARG, "edges must be strictly increasing");
     int rc = finish_update(ctx);
     if (rc) return rc;
-    // the edges in the state precision and the cleared sums in one upload, to a
-    // buffer the context keeps (an allocation per call cost 200 us: the pool
-    // gave its memory back at every synchronisation)
+    // the cleared sums (and room for the error word) and the edges in the state
+    // precision in one upload, to a buffer the context keeps (an allocation per
+    // call cost 200 us: the pool gave its memory back at every synchronisation)
     const bool f32 = ctx->prec == M2M_FP32C;
-    const size_t ob = 32 * (size_t)nshell, eb = (f32 ? 4 : 8) * (size_t)(nshell + 1);
+    const size_t sb = 32 * (size_t)nshell, ob = sb + 8, eb = (f32 ? 4 : 8) * (size_t)(nshell + 1);
     if (ctx->vm_bytes < ob + eb) {
         CU(cudaStreamSynchronize(ctx->st));
         if (ctx->d_vm) cudaFree(ctx->d_vm);
@@ -1439,7 +1439,7 @@ int m2m_velocity_moments(m2m_ctx *ctx, const double *r2_edges, int32_t nshell, d
     cudaError_t e = cudaMemcpyAsync(dout, up.data(), ob + eb, cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess) {
         const int copies = vmoments_copies(nshell);
-        const size_t sm = ob * copies + eb;
+        const size_t sm = sb * copies + eb;
         int g = ctx->nsm * 4;
         long long need = (ctx->n + 255) / 256;
         if (g > need) g = (int)need;
@@ -1447,17 +1447,21 @@ int m2m_velocity_moments(m2m_ctx *ctx, const double *r2_edges, int32_t nshell, d
             k_vmoments<float><<<g, 256, sm, ctx->st>>>((const float *)ctx->x, (const float *)ctx->y, (const float *)ctx->z,
                                                         (const float *)ctx->vx, (const float *)ctx->vy,
                                                         (const float *)ctx->vz, ctx->w, ctx->n, (const float *)de,
-                                                        nshell, copies, dout);
+                                                        nshell, copies, dout, ctx->d_err);
         else
             k_vmoments<double><<<g, 256, sm, ctx->st>>>((const double *)ctx->x, (const double *)ctx->y,
                                                          (const double *)ctx->z, (const double *)ctx->vx,
                                                          (const double *)ctx->vy, (const double *)ctx->vz, ctx->w,
-                                                         ctx->n, (const double *)de, nshell, copies, dout);
+                                                         ctx->n, (const double *)de, nshell, copies, dout, ctx->d_err);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, ob, cudaMemcpyDeviceToHost, ctx->st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(up.data(), dout, ob, cudaMemcpyDeviceToHost, ctx->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->st);
     if (e != cudaSuccess) return set_err(ctx, M2M_ERR_CUDA, "velocity moments: %s", cudaGetErrorString(e));
-    return check_err_word(ctx);
+    memcpy(out, up.data(), sb);
+    int h = 0;
+    memcpy(&h, up.data() + sb, 4);
+    return err_word(ctx, h);
 }
 
 // ---------------------------------------------------------------- shards
