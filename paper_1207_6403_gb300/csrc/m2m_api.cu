@@ -22,6 +22,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <string>
 #include <tuple>
@@ -1167,15 +1168,17 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         if (lay) kfns.push_back(pass_kernel_f32_pipe(lay));
         for (int pk : {PK_ANY, PK_HERNQUIST, PK_LOG, PK_SH, PK_HERNQUIST_NFW, PK_SH_TRI, PK_SH_FULL})
                 for (int fl : {F_STEADY, F_STEADY | F_MINMAX, F_PUSH | F_SCAT | F_STATS,
-                               F_PUSH | F_SCAT | F_STATS | F_MINMAX, F_CELLS | F_UPD})
+                               F_PUSH | F_SCAT | F_STATS | F_MINMAX, F_CELLS | F_UPD, F_SCAT | F_STATS, (int)F_UPD})
                     if (void *f = pass_kernel_f32_compiled(fl, lay, pk)) kfns.push_back(f);
         if (lay) kfns.push_back(pass_kernel_f32_pipe_steady(lay));
         kfns.push_back(pass_kernel_f32_batch(lay));
-        if (lay) kfns.push_back(pass_kernel_f32_batch(lay, true));
-        if (lay == 2) kfns.push_back(pass_kernel_f32_batch(lay, true, PK_HERNQUIST_NFW));
+        for (int fl : {(int)F_STEADY, (int)F_UPD})
+            for (int pk : {PK_ANY, PK_HERNQUIST_NFW}) kfns.push_back(pass_kernel_f32_batch(lay, fl, pk));
         for (int pk : {PK_HERNQUIST, PK_LOG, PK_HERNQUIST_NFW})
             for (bool solo : {false, true}) kfns.push_back(steps_kernel_f32(lay, pk, solo));
     }
+    std::sort(kfns.begin(), kfns.end());         // (one kernel serves several signatures)
+    kfns.erase(std::unique(kfns.begin(), kfns.end()), kfns.end());
     for (void *f : kfns) {
         if (!f) continue;                    // no such variant compiled
         cudaFuncAttributes fa;
@@ -2010,8 +2013,9 @@ int batch_pass(m2m_batch *b, int flags, int cache_read, int half, long long rec_
     bp.rec_step = rec_step;
     bp.step = b->d_step;
     void *args[] = {&bp};
-    const bool steady = flags == F_STEADY && cache_read;
-    cudaError_t e = launch_dependent(pass_kernel_f32_batch(b->layout, steady, b->pk), dim3(b->pgrid), dim3(1024), args,
+    // (the compiled passes read and write the cells)
+    const int fl = (flags == F_STEADY || flags == F_UPD) && cache_read ? flags : 0;
+    cudaError_t e = launch_dependent(pass_kernel_f32_batch(b->layout, fl, b->pk), dim3(b->pgrid), dim3(1024), args,
                                      batch_smem(b, flags), b->st);
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "batched pass: %s", cudaGetErrorString(e));
     return M2M_OK;

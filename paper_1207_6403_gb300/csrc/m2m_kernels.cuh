@@ -1743,7 +1743,7 @@ void *pass_kernel_f32_pipe(int layout);
 void *pass_kernel_f32_steady(int layout, int pk = PK_ANY);
 void *pass_kernel_f32_compiled(int flags, int layout, int pk);   // NULL if not compiled
 void *pass_kernel_f32_pipe_steady(int layout);
-void *pass_kernel_f32_batch(int layout, bool steady = false, int pk = PK_ANY);
+void *pass_kernel_f32_batch(int layout, int flags = 0, int pk = PK_ANY);   // flags compiled in, or run-time flags
 void *steps_kernel_f32(int layout, int pk, bool solo);                      // NULL if not compiled
 void *pass_kernel_f64(int threads, int layout);
 void *cells_kernel_f32();

@@ -24,24 +24,24 @@ void *pass_kernel_f32_pipe_steady(int layout) {
 }
 
 // All models of a batch in one launch (compiled layouts, plain loads); the
-// steady-state step with its flags compiled in.
-void *pass_kernel_f32_batch(int layout, bool steady, int pk) {
-    if (steady) {
-        // the batched trial-potential models: Hernquist stars in Hernquist + NFW
-        if (layout == 2 && pk == PK_HERNQUIST_NFW) return (void *)k_pass_batch<float, 1024, 1, 2, F_STEADY, PK_HERNQUIST_NFW>;
-        switch (layout) {
-            case 1: return (void *)k_pass_batch<float, 1024, 1, 1, F_STEADY>;
-            case 2: return (void *)k_pass_batch<float, 1024, 1, 2, F_STEADY>;
-            case 3: return (void *)k_pass_batch<float, 1024, 1, 3, F_STEADY>;
-            case 4: return (void *)k_pass_batch<float, 1024, 1, 4, F_STEADY>;
-            default: break;
-        }
-    }
+// steady-state step and the update-only pass with their flags compiled in.
+template <int L>
+static void *batch_layout(int flags, int pk) {
+    // the batched trial-potential models: Hernquist stars in Hernquist + NFW
+    if constexpr (L == 2)
+        if (flags == F_STEADY && pk == PK_HERNQUIST_NFW)
+            return (void *)k_pass_batch<float, 1024, 1, 2, F_STEADY, PK_HERNQUIST_NFW>;
+    if (flags == F_STEADY) return (void *)k_pass_batch<float, 1024, 1, L, F_STEADY>;
+    if (flags == F_UPD) return (void *)k_pass_batch<float, 1024, 1, L, F_UPD>;
+    return (void *)k_pass_batch<float, 1024, 1, L>;
+}
+
+void *pass_kernel_f32_batch(int layout, int flags, int pk) {
     switch (layout) {
-        case 1: return (void *)k_pass_batch<float, 1024, 1, 1>;
-        case 2: return (void *)k_pass_batch<float, 1024, 1, 2>;
-        case 3: return (void *)k_pass_batch<float, 1024, 1, 3>;
-        case 4: return (void *)k_pass_batch<float, 1024, 1, 4>;
+        case 1: return batch_layout<1>(flags, pk);
+        case 2: return batch_layout<2>(flags, pk);
+        case 3: return batch_layout<3>(flags, pk);
+        case 4: return batch_layout<4>(flags, pk);
         default: return (void *)k_pass_batch<float, 1024, 1, 0>;
     }
 }
