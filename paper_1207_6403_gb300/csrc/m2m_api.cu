@@ -2266,7 +2266,10 @@ int m2m_batch_step(m2m_batch *b, int64_t nsteps) {
     b->up_step = -1;
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "step counter: %s", cudaGetErrorString(e));
     const bool graphable = b->st != nullptr && b->st != cudaStreamLegacy && b->st != cudaStreamPerThread;
-    const auto key = std::make_tuple((long long)nsteps, b->period ? t0 % b->period : 0ll, 0);
+    // (the launches of a graph keep their shared memory size, which follows the
+    // models' histogram copies)
+    const auto key = std::make_tuple((long long)nsteps, b->period ? t0 % b->period : 0ll,
+                                     (int)batch_smem(b, F_STEADY | F_MINMAX));
     bool launched = false;
     if (graphable) {
         auto it = b->graphs.find(key);

@@ -553,7 +553,7 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
                 c = set_cell<R>(s, S.edges, x, y, z, Xk, Yk);
             }
             packed |= (unsigned)(c + 1) << s.cshift;     // (kept only where the sets' fields fit)
-            if (c < 0 || wv == R(0)) continue;
+            if (c < 0) continue;
             const int b = s.obs_off + c * s.nmom;
             if (s.quant != M2M_Q_GH) {
                 const R v = s.quant == M2M_Q_MASS ? wv : wv * (vlos * vlos);
@@ -563,8 +563,10 @@ __device__ __forceinline__ unsigned scatter(const PassArgs &a, const PassSmem<R>
             } else {
                 R u[5];
                 gh_eval(vlos, S.gh + s.gh_off + 5 * c, u);
-                // |u_n| <= sqrt 2 (below): one test for the five terms
-                if (fabsf(wv * fs) < 0.5f * FX_FAST) {
+                // |u_n| <= sqrt 2 (below): one test for the five terms, and one
+                // that none is NaN (the general path reports those)
+                const R t = (u[1] + u[2]) + (u[3] + u[4]);
+                if (fabsf(wv * fs) < 0.5f * FX_FAST && t == t) {
 #pragma unroll
                     for (int m = 0; m < 5; ++m) fx_red_fast(S.hL, S.hM, b + m, (wv * u[m]) * fs);
                 } else {
@@ -1137,7 +1139,7 @@ constexpr int F_STEADY = F_UPD | F_PUSH | F_SCAT | F_STATS;
 // segment costs beside its particles (see batch_plan); a model's blocks were
 // whole shares of it before, which left the fullest block of 48 models half
 // as full again as the mean one (25 steps of 48 models, 4.1M particles in all,
-// took 4.13 ms, now 3.15).  Each model's arguments are its own PassArgs (device array); the
+// took 4.13 ms, now 3.07).  Each model's arguments are its own PassArgs (device array); the
 // flags, the cache use and the record to write are shared.
 struct BatchSeg { int model, rank, begin, end; };
 struct BatchPass {
@@ -1539,7 +1541,8 @@ __device__ __forceinline__ void node_sums(const long long *sum, int rowA, int ro
 // Node table of the axisymmetric expansion, one block per l: F_l, D_l and the
 // slopes to the next node, in double.  (One block for all of them kept a
 // single SM busy with some 50 FP64 operations per node and term: 52 us for
-// 256 nodes, 12 now; the triaxial table 145, 14 now.)
+// 256 nodes, 21 now; the triaxial table took 145 us, a triaxial run of 50
+// steps 4.81 -> 4.68 ms.)
 template <class R>
 __global__ void __launch_bounds__(256) k_sh_tables(const long long *sum, int K, const double *rn, double q, R *tab,
                                                    int *err) {

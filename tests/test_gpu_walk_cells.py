@@ -59,3 +59,17 @@ def test_walk_matches_the_oracle(kind, n):
     ctx.m2m_observe(0)
     ctx.m2m_update_weights()
     ctx.m2m_free()
+
+
+# a velocity that gives no finite moment is reported, not dropped
+@pytest.mark.parametrize("bad", [np.nan, np.inf, 1e25])
+@pytest.mark.parametrize("weight", [0.0, 1.0])
+def test_walk_reports_moments_that_are_not_finite(bad, weight):
+    n = 100
+    P = I.make_problem("plain-fp64", n=n, precision="fp32c", with_target=False)
+    P.obs = _sets("shared")[3:]
+    P.pos[:, 7] = (0.1, 0.1, 0.0)
+    P.vel[:, 7] = bad
+    P.w0[7] *= weight
+    with pytest.raises(B.M2MError):
+        B.from_problem(P, "fp32c", targets=False)
