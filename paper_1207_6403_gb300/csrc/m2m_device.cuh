@@ -309,39 +309,6 @@ __device__ __forceinline__ void fixed_add(unsigned *lo, unsigned *hi, int b, lon
 // ------------------------------------------------------------ potentials
 template <class R> struct Acc3 { R x, y, z; };
 
-// Correctly rounded double division and square root for the FP64 force, in
-// as few FP64 operations as the method allows (the pipe that bounds the pass):
-// the hardware's 20-bit reciprocal (root) approximation, one third-order
-// step, and Markstein's final correction with the exact remainder (P. W.
-// Markstein, IBM J. Res. Dev. 34 (1990) 111): q + (a - q b) y rounds to a/b
-// when q is within an ulp of it and y is 1/b to within rounding.  6 and 9
-// operations.  Operands outside 2^-500 .. 2^500 (zeros, NaN, infinities) take
-// the language's operations.
-__device__ __forceinline__ bool mid_range(double v) {
-    return (((unsigned)__double2hiint(v) >> 20) & 0x7ffu) - 523u <= 1000u;
-}
-__device__ __forceinline__ double div_rn(double a, double b) {
-    if (!(mid_range(a) && mid_range(b))) return a / b;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    const double e = fma(-b, y, 1.0);
-    y = fma(y, fma(e, e, e), y);
-    const double q = a * y;
-    return fma(fma(-b, q, a), y, q);
-}
-__device__ __forceinline__ double sqrt_rn(double a) {
-    if (!(mid_range(a) && __double2hiint(a) >= 0)) return sqrt(a);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-    double g = a * y, h = 0.5 * y;
-    const double e = fma(-g, h, 0.5), c = fma(1.5 * e, e, e);     // g = sqrt(a)(1 - e) to first order
-    g = fma(g, c, g);
-    h = fma(h, c, h);
-    return fma(fma(-g, g, a), h, g);
-}
-__device__ __forceinline__ float div_rn(float a, float b) { return a / b; }
-__device__ __forceinline__ float sqrt_rn(float a) { return sqrtf(a); }
-
 __device__ __forceinline__ float nfw_f(float r, const PotDev &p) {
     // M(r)/r^3, M = C [ln(1+u) - u/(1+u)], u = r/r_s
     float u = r * p.cf[2];
@@ -360,10 +327,10 @@ __device__ __forceinline__ double nfw_f(double r, const PotDev &p) {
     if (u < 1e-3) {
         mu = u * u * (0.5 - u * (2.0 / 3.0 - u * (0.75 - 0.8 * u)));
     } else {
-        mu = log1p(u) - div_rn(u, 1.0 + u);
+        mu = log1p(u) - u / (1.0 + u);
     }
     double r3 = r * r * r;
-    return r > 0. ? div_rn(p.c[0] * mu, r3) : 0.;
+    return r > 0. ? p.c[0] * mu / r3 : 0.;
 }
 
 // ------------------------------------------------------------ multipoles
@@ -729,9 +696,9 @@ template <class R>
 __device__ __forceinline__ void acc_hernquist(R x, R y, R z, const PotDev &p, Acc3<R> &g) {
     R GM = KC(R, p.c[0], p.cf[0]), aa = KC(R, p.c[1], p.cf[1]);
     R r2 = (x * x + y * y) + z * z;
-    R r = sqrt_rn(r2);
+    R r = sqrt(r2);
     R s = r + aa;
-    R f = r2 > R(0) ? div_rn(GM, (r * s) * s) : R(0);
+    R f = r2 > R(0) ? GM / ((r * s) * s) : R(0);
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-(f * z));
@@ -741,7 +708,7 @@ __device__ __forceinline__ void acc_log(R x, R y, R z, const PotDev &p, Acc3<R> 
     R Rc2 = KC(R, p.c[0], p.cf[0]), iq2 = KC(R, p.c[1], p.cf[1]), v0sq = KC(R, p.c[2], p.cf[2]);
     R R2 = x * x + y * y;
     R D = (Rc2 + R2) + (z * z) * iq2;
-    R f = div_rn(v0sq, D);
+    R f = v0sq / D;
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-((f * iq2) * z));
@@ -749,7 +716,7 @@ __device__ __forceinline__ void acc_log(R x, R y, R z, const PotDev &p, Acc3<R> 
 template <class R>
 __device__ __forceinline__ void acc_nfw(R x, R y, R z, const PotDev &p, Acc3<R> &g) {
     R r2 = (x * x + y * y) + z * z;
-    R f = nfw_f(sqrt_rn(r2), p);
+    R f = nfw_f(sqrt(r2), p);
     g.x = g.x + (-(f * x));
     g.y = g.y + (-(f * y));
     g.z = g.z + (-(f * z));
@@ -762,9 +729,9 @@ template <class R>
 __device__ __forceinline__ Acc3<R> acc1_hernquist(R x, R y, R z, const PotDev &p) {
     R GM = KC(R, p.c[0], p.cf[0]), aa = KC(R, p.c[1], p.cf[1]);
     R r2 = (x * x + y * y) + z * z;
-    R r = sqrt_rn(r2);
+    R r = sqrt(r2);
     R s = r + aa;
-    R f = r2 > R(0) ? div_rn(GM, (r * s) * s) : R(0);
+    R f = r2 > R(0) ? GM / ((r * s) * s) : R(0);
     return Acc3<R>{-(f * x), -(f * y), -(f * z)};
 }
 template <class R>
@@ -772,7 +739,7 @@ __device__ __forceinline__ Acc3<R> acc1_log(R x, R y, R z, const PotDev &p) {
     R Rc2 = KC(R, p.c[0], p.cf[0]), iq2 = KC(R, p.c[1], p.cf[1]), v0sq = KC(R, p.c[2], p.cf[2]);
     R R2 = x * x + y * y;
     R D = (Rc2 + R2) + (z * z) * iq2;
-    R f = div_rn(v0sq, D);
+    R f = v0sq / D;
     return Acc3<R>{-(f * x), -(f * y), -((f * iq2) * z)};
 }
 

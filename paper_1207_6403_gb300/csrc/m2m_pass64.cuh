@@ -13,8 +13,7 @@
 //  - cells are decided on the doubles' bit patterns (order-preserving integer
 //    keys, exactly the double comparisons) and the float index guess comes
 //    from the bits, so a bin search has no FP64 instruction;
-//  - an expansion's force is a call (m2m_device.cuh, ex_accel_call) and the
-//    force's quotient and root are the short forms div_rn and sqrt_rn;
+//  - an expansion's force is a call (m2m_device.cuh, ex_accel_call);
 //  - exp is table driven (P. T. P. Tang, ACM TOMS 15 (1989) 144: exp(x) =
 //    2^(k/128) exp(r), |r| <= ln 2/256, a quintic in r), 10 operations; the
 //    weight's exp(d) is 1 + its series for |d| < 2^-10;
