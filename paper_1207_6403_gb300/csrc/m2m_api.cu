@@ -135,7 +135,7 @@ struct m2m_ctx {
     int test_stall = 0;              // test only: the next launch's block 0 skips its first arrival
     long long test_wait_ns = 0;      //   and its barrier waits are limited to this
     // FP64: what a pass leaves for the next one of the same m2m_step call
-    // ([6][n]: ln(w/w_hat), m, Gaussian factor, force), and which of it holds
+    // ([7][n]: ln(w/w_hat) and its rest, m, Gaussian factor, force), and which of it holds
     double *d_c64 = nullptr, *d_exp = nullptr;
     bool in_step = false, c64_lnw = false, c64_gh = false, c64_force = false;
     void *d_vm = nullptr;            // velocity moments: sums and shell edges
@@ -398,10 +398,11 @@ void fill_args(const m2m_ctx *c, PassArgs &a, int flags) {
     a.exp_tab = c->d_exp;
     if (c->in_step && c->d_c64) {
         a.c64_lnw = c->d_c64;
-        if (c->layout == 1 || c->layout == 2) { a.c64_m = c->d_c64 + c->n; a.c64_g = c->d_c64 + 2 * c->n; }
+        a.c64_lnl = c->d_c64 + c->n;
+        if (c->layout == 1 || c->layout == 2) { a.c64_m = c->d_c64 + 2 * c->n; a.c64_g = c->d_c64 + 3 * c->n; }
         a.c64_read = (c->c64_lnw ? C64_LNW : 0) | (c->c64_gh ? C64_GH : 0);
         if (!c->sh_on) {
-            a.facc = c->d_c64 + 3 * c->n;
+            a.facc = c->d_c64 + 4 * c->n;
             a.facc_read = (flags & F_PUSH) && c->c64_force;
         }
     }
@@ -1091,8 +1092,8 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         // only where it leaves the caller most of the memory; without it every
         // pass computes these values itself
         size_t freeb = 0, totb = 0;
-        if (cudaMemGetInfo(&freeb, &totb) == cudaSuccess && 48 * (size_t)n < freeb / 4 &&
-            cudaMalloc((void **)&ctx->d_c64, 48 * (size_t)n) != cudaSuccess)
+        if (cudaMemGetInfo(&freeb, &totb) == cudaSuccess && C64_BYTES * (size_t)n < freeb / 4 &&
+            cudaMalloc((void **)&ctx->d_c64, C64_BYTES * (size_t)n) != cudaSuccess)
             ctx->d_c64 = nullptr;
         cudaGetLastError();
     }

@@ -21,7 +21,7 @@ constexpr int MAXCELLS = 16385;
 enum { F_UPD = 1, F_PUSH = 2, F_SCAT = 4, F_STATS = 8, F_MINMAX = 16, F_CELLS = 32 };
 enum { G_LIN = 0, G_LOG = 1, G_BIS = 2 };
 enum { REC_EVERY = 2 };
-enum { C64_LNW = 1, C64_GH = 2 };
+enum { C64_LNW = 1, C64_GH = 2, C64_BYTES = 56 };    // C64_BYTES: per particle, all that is kept
 enum { ERR_NONFINITE = 1, ERR_OVERFLOW = 2, ERR_TIMEOUT = 4 };
 
 struct SetDev {
@@ -94,7 +94,8 @@ struct PassArgs {
     const void *sh_tab; int sh_K, sh_row;   // expansion node table (R, sh_row values per node) or NULL
     // FP64, inside one m2m_step call: what the preceding pass left for the same
     // particles ([n] each, or null), and which of it holds (C64_* bits)
-    double *c64_lnw, *c64_m, *c64_g;        // ln(w/w_hat); m and the Gaussian factor of the GH cell
+    double *c64_lnw, *c64_lnl;              // ln(w/w_hat), rounded and the rest
+    double *c64_m, *c64_g;                  // m and the Gaussian factor of the GH cell
     int c64_read;
     const double *exp_tab;                  // FP64: 2^(j/128)
     void *facc; int facc_read;              // expansion potentials: force at the positions (R, [3][n]) or NULL

@@ -6,17 +6,17 @@
 // step's own and take a twentieth of the time).  What follows from that:
 //  - inside one m2m_step call a pass leaves what the next one would compute
 //    again from the same particle: the force at the new position, ln(w/w_hat)
-//    of the stored weight and, per Gauss-Hermite set, m and the Gaussian
-//    factor of the cell the scatter found (48 bytes per particle, PassArgs
-//    c64); m2m_step alone sets the flags, so a caller may change its arrays
-//    between calls as before;
+//    of the stored weight (see log_carry) and, per Gauss-Hermite set, m and
+//    the Gaussian factor of the cell the scatter found (56 bytes per particle,
+//    PassArgs c64); m2m_step alone sets the flags, so a caller may change its
+//    arrays between calls as before;
 //  - cells are decided on the doubles' bit patterns (order-preserving integer
 //    keys, exactly the double comparisons) and the float index guess comes
 //    from the bits, so a bin search has no FP64 instruction;
 //  - an expansion's force is a call (m2m_device.cuh, ex_accel_call);
 //  - exp is table driven (P. T. P. Tang, ACM TOMS 15 (1989) 144: exp(x) =
 //    2^(k/128) exp(r), |r| <= ln 2/256, a quintic in r), 10 operations; the
-//    weight's exp(d) is 1 + its series for |d| < 2^-10;
+//    weight's exp(d) is 1 + its series to d^8 for |d| < 2^-5 (the rest is below 2^-63);
 //  - the moments are polynomials of m with the constants of gh_record, no
 //    division;
 //  - a double shared-memory add is a compare-and-swap loop, which the lanes
@@ -127,6 +127,33 @@ __device__ __forceinline__ GhPoint gh_point(const double *r, double vlos, const 
     return {m, r[3] * exp_neg((dv * m) * r[2], T)};
 }
 
+// A weight far enough from the ends of the double range for log_carry.
+__device__ __forceinline__ bool mid_weight(double w) {
+    return ((unsigned)__double2hiint(w) >> 20) - 123u <= 1800u;          // 2^-900 .. 2^900
+}
+
+// ln(wn/w_hat) of the stored weight wn = w + w e (rounded; e = e^d - 1) from
+// ln(w/w_hat) = L + l: L + d less what the rounding of wn took, rem/wn, as a
+// sum and its remainder l (T. J. Dekker, Numer. Math. 18 (1971) 224, the
+// larger term first by exponent).  L + d alone would not do: its roundings
+// and the weights' add up over the steps of a call, and a weight that no
+// longer moves (|d| below half an ulp) would leave the sum moving on.  As it
+// is, the error after 4000 steps is that of one fresh logarithm (rms 6e-17;
+// L + d alone 5e-15 and more).  Seven FP64 operations, where the quotient and
+// the logarithm take 40: 300,000 particles, pixels + apertures, 25 steps 2820
+// us; with the series and so the carry only below |d| = 2^-10, where half of
+// the warps have a lane beyond it, 3210.
+__device__ __forceinline__ double log_carry(double L, double &l, double w, double wn, double d, double e) {
+    const double rem = fma(w, e, w - wn);            // the difference is exact (|e| < 2^-4)
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(wn));               // 20 bits: rem is below an ulp
+    const double c = d + (l - rem * y);
+    const bool first = ((unsigned)__double2hiint(L) & 0x7fffffffu) >= ((unsigned)__double2hiint(c) & 0x7fffffffu);
+    const double p = first ? L : c, q = first ? c : L, s = p + q;
+    l = q - (s - p);
+    return s;
+}
+
 // One pass over the particles of block `bid` of `nblk`.  L: compiled layout
 // (1: pixels + apertures, 2: shells + GH annuli, 3: shells + mass and v^2
 // annuli), 0: the run-time set walk.
@@ -219,10 +246,10 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
         double wn = w;
         if (fl & (F_UPD | F_STATS)) {
             if (d_pos(w)) {
-                double Lw;
-                if (a.c64_read & C64_LNW) Lw = a.c64_lnw[i];
+                double Lw, Ll = 0.0;          // ln(w/w_hat) and, kept, what its rounding left out
+                if (a.c64_read & C64_LNW) { Lw = a.c64_lnw[i]; Ll = a.c64_lnl[i]; }
                 else Lw = log(w / a.what[i]);
-                double wr = w;
+                double wr = w, Lk = Lw;       // Lk: what the next pass finds
                 if (fl & F_UPD) {
                     double dot = 0.0;
                     if constexpr (L == 0) {
@@ -273,15 +300,24 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
                     }
                     const double G = a.mu * (-Lw - a.ent_c) - dot;
                     const double d = a.eps_dt * G;
-                    if (((unsigned)__double2hiint(d) & 0x7fffffffu) < 0x3F500000u) {    // |d| < 2^-10
-                        double e = fma(d, 1.0 / 24.0, 1.0 / 6.0);
+                    const bool small = ((unsigned)__double2hiint(d) & 0x7fffffffu) < 0x3FA00000u;   // |d| < 2^-5
+                    double e = 0.0;
+                    if (small) {
+                        e = fma(d, 1.0 / 40320.0, 1.0 / 5040.0);
+                        e = fma(d, e, 1.0 / 720.0);
+                        e = fma(d, e, 1.0 / 120.0);
+                        e = fma(d, e, 1.0 / 24.0);
+                        e = fma(d, e, 1.0 / 6.0);
                         e = fma(d, e, 0.5);
                         e = fma(d, e, 1.0);
-                        wn = fma(w, d * e, w);
+                        e = d * e;                               // e^d - 1
+                        wn = fma(w, e, w);
                     } else {
                         wn = w * exp(d);
                     }
                     wr = wn;
+                    if (a.c64_lnw && small && mid_weight(wn)) Lk = log_carry(Lw, Ll, w, wn, d, e);
+                    else if (a.c64_lnw) { Lk = log(wn / a.what[i]); Ll = 0.0; }
                     Lw = Lw + d;
                     if (d_bad(wn)) bad = true;
                 }
@@ -289,7 +325,7 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
                     s_d = fma(-wr, Lw, s_d);
                     w_d += wr;
                 }
-                if (a.c64_lnw) a.c64_lnw[i] = Lw;
+                if (a.c64_lnw) { a.c64_lnw[i] = Lk; a.c64_lnl[i] = Ll; }
             } else if (__double_as_longlong(w) != 0ll) {
                 bad = true;       // negative, -0 or NaN weight
             }
