@@ -16,6 +16,12 @@ __device__ __forceinline__ double rcp_d(double d) {
     return fma(y, fma(e, e, e), y);
 }
 
+// 0, or a magnitude between 2^-400 and 2^400 (on the bits: no FP64 instruction).
+__device__ __forceinline__ bool square_ok(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu;
+    return (hi >> 20) - 623u <= 800u || (hi | (unsigned)__double2loint(v)) == 0u;
+}
+
 // Float -> double exactly, with integer instructions for normal numbers (the
 // conversion instruction runs on the FP64 pipe).
 __device__ __forceinline__ double widen(float f) {
@@ -70,13 +76,15 @@ __global__ void __launch_bounds__(256) k_vmoments(const R *x, const R *y, const 
         const double R2 = fma(X, X, Y * Y), r2 = fma(Z, Z, R2);
         const double s = fma(X, U, fma(Y, V, Z * W)), t = fma(X, V, -(Y * U));
         const double v2 = fma(U, U, fma(V, V, W * W));
-        // (on the axis v_phi = 0, at the centre v_r = 0 too)
-        const bool safe = R2 > 1e-100 && r2 < 1e100;
+        // (where a square would leave the double range, the quotients before
+        // the squares; on the axis v_phi = 0, at the centre v_r = 0 too)
+        const bool safe = R2 > 1e-100 && r2 < 1e100 && square_ok(s) && square_ok(t);
         const double k = rcp_d(safe ? r2 * R2 : 1.0);
         double vr2 = (s * s) * (R2 * k), vp2 = (t * t) * (r2 * k);
         if (!safe) {
-            vr2 = r2 > 0 ? s * s / r2 : 0.0;
-            vp2 = R2 > 0 ? t * t / R2 : 0.0;
+            const double vr = r2 > 0 ? s / sqrt(r2) : 0.0, vp = R2 > 0 ? t / sqrt(R2) : 0.0;
+            vr2 = vr * vr;
+            vp2 = vp * vp;
         }
         double *o = mine + 4 * lo * copies;
         atomicAdd(o, wi);
