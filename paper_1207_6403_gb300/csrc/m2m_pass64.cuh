@@ -43,11 +43,15 @@ __device__ __forceinline__ long long dkey(double v) {
     return (b << 1) == 0 ? 0ll : b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-// The float nearest a double towards zero, from its bits (0 below the float
-// range, infinite above).
+// The float nearest a double towards zero, from its bits (infinite above the
+// float range; integer instructions only, also for subnormal floats).
 __device__ __forceinline__ float d2f_bits(double v) {
-    const unsigned s = (unsigned)__double2hiint(v) & 0x80000000u;
-    return __uint_as_float(__float_as_uint(d2f_fast(fabs(v))) | s);
+    const unsigned hi = (unsigned)__double2hiint(v);
+    const int e = (int)((hi >> 20) & 0x7ffu) - 896;                     // float biased exponent
+    const unsigned m = __funnelshift_l((unsigned)__double2loint(v), hi, 3) & 0x7fffffu;
+    unsigned r = e > 0 ? ((unsigned)e << 23) | m : __funnelshift_rc(m | 0x800000u, 0u, (unsigned)(1 - e));
+    r = e >= 255 ? 0x7f800000u : r;
+    return __uint_as_float(r | (hi & 0x80000000u));
 }
 
 // find_fast on keys: the guess is within a cell of the true one, the keys of
