@@ -52,7 +52,6 @@ struct LaunchShape {
 struct m2m_ctx {
     int prec;
     long long n;
-    long long launch_n;  // particles of one launch: n, in a batch those of all its models
     void *x, *y, *z, *vx, *vy, *vz;
     double *w, *what;
     cudaStream_t st;
@@ -253,12 +252,13 @@ size_t pass_smem_copies(const m2m_ctx *c, int flags, int hrep) {
 // keep fewer.  Measured, 1 / 8 / 32 copies: 8M particles in their own
 // spherical-harmonic potential, 50 steps, 10.88 / 10.47 / 10.42 ms; 48 models
 // of 4.1M particles in all, 25 steps, 4.17 / 4.07 / 3.99 ms; 1M particles,
-// 25 steps, 774 / 767 / 777 us.
-int hist_copies(const m2m_ctx *c) {
+// 25 steps, 774 / 767 / 777 us.  launch_n: particles of the launch, in a fused
+// batch those of all its models.
+int hist_copies(const m2m_ctx *c, long long launch_n) {
     // the kernels' static shared memory, and a solo residual's arrays
     const size_t room = (size_t)c->smem_optin - 4096 - (c->nobs <= SOLO_OBS ? 16 * (size_t)c->nobs : 0);
     if (c->prec == M2M_FP32C && (c->threads != 1024 || c->pipe || (c->layout != 2 && c->layout != 3))) return 1;
-    int r = c->launch_n >= 8ll * 1024 * c->nsm ? 32 : 8;
+    int r = launch_n >= 8ll * 1024 * c->nsm ? 32 : 8;
     if (c->prec == M2M_FP64) {
         // (r - 1) nobs FP64 adds when a block sums the copies: at most a
         // fiftieth of its particles' some 180 operations
@@ -269,7 +269,9 @@ int hist_copies(const m2m_ctx *c) {
     return r;
 }
 
-size_t pass_smem(const m2m_ctx *c, int flags) { return pass_smem_copies(c, flags, hist_copies(c)); }
+size_t pass_smem(const m2m_ctx *c, int flags, long long launch_n) {
+    return pass_smem_copies(c, flags, hist_copies(c, launch_n));
+}
 
 // Pixels of grid set g0 -> cell of grid set g1, when every edge of g1 is an
 // edge of g0 as the floats the cells are decided against (the smallest
@@ -361,7 +363,7 @@ LaunchShape pick_kernel(const m2m_ctx *c) {
     return {pass_kernel_f64(nt, c->layout), nt};
 }
 
-void fill_args(const m2m_ctx *c, PassArgs &a, int flags) {
+void fill_args(const m2m_ctx *c, PassArgs &a, int flags, long long launch_n) {
     memset(&a, 0, sizeof a);
     a.x = c->x; a.y = c->y; a.z = c->z; a.vx = c->vx; a.vy = c->vy; a.vz = c->vz;
     a.w = c->w; a.what = c->what; a.lnwhat = c->d_lnwhat; a.n = c->n; a.flags = flags;
@@ -379,7 +381,7 @@ void fill_args(const m2m_ctx *c, PassArgs &a, int flags) {
     a.gh_tab = c->d_gh; a.gh_len = c->gh_len;
     a.coef = c->d_coef_r;
     a.slots = c->d_slots; a.fx_shift = c->fx_shift; a.y_acc = c->d_y_acc; a.fx_atomic = c->fx_atomic;
-    a.hrep = hist_copies(c);
+    a.hrep = hist_copies(c, launch_n);
     a.cell_shift = c->cell_shift;
     a.stat_slots = c->d_stat_slots + (size_t)2 * c->slot_cap * c->stat_par;
     a.rec_pending = c->rec_pending; a.rec_write_ring = 1; a.rec_step = c->rec_step;
@@ -445,9 +447,9 @@ int potential_signature(const m2m_ctx *c) {
 
 int launch_pass(m2m_ctx *ctx, int flags, int *grid_out = nullptr) {
     PassArgs a;
-    fill_args(ctx, a, flags);
+    fill_args(ctx, a, flags, ctx->n);
     LaunchShape ks = pick_kernel(ctx);
-    size_t sm = pass_smem(ctx, flags);
+    size_t sm = pass_smem(ctx, flags, ctx->n);
     int occ = 0;
     if (ctx->pipe && ctx->prec == M2M_FP32C && ctx->threads == 1024 && ctx->layout != 0) {
         // block-level bulk-copy pipeline when its stage buffers fit beside the tables
@@ -567,7 +569,7 @@ void *persistent_kernel(m2m_ctx *ctx, long long m, size_t *smem_out, int *grid_o
         return nullptr;
     void *fn = steps_kernel_f32(ctx->layout, potential_signature(ctx), false);
     if (!fn) return nullptr;
-    size_t sm = pass_smem(ctx, F_STEADY);
+    size_t sm = pass_smem(ctx, F_STEADY, ctx->n);
     *solo_out = false;
     if (m >= 3 && ctx->nobs <= SOLO_OBS && sm + 16 * (size_t)ctx->nobs + 4096 <= (size_t)ctx->smem_optin)
         if (void *fs = steps_kernel_f32(ctx->layout, potential_signature(ctx), true)) {
@@ -597,7 +599,7 @@ int launch_steps(m2m_ctx *ctx, void *fn, size_t sm, int grid, bool solo, long lo
     if (rc0) return rc0;
     StepsArgs A;
     memset(&A, 0, sizeof A);
-    fill_args(ctx, A.p, F_STEADY);
+    fill_args(ctx, A.p, F_STEADY, ctx->n);
     A.p.cache_write = 1;
     A.p.rec_pending = 0;
     ResArgs &r = A.r;
@@ -877,7 +879,6 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
     ctx = new m2m_ctx();   // value-initialised: all pointers NULL
     ctx->prec = precision;
     ctx->n = n;
-    ctx->launch_n = n;
     ctx->x = x; ctx->y = y; ctx->z = z; ctx->vx = vx; ctx->vy = vy; ctx->vz = vz;
     ctx->w = w; ctx->what = what;
     ctx->st = (cudaStream_t)stream;
@@ -1682,7 +1683,7 @@ int m2m_get_cells(m2m_ctx *ctx, int32_t *obs_cells, int32_t *prior_cells) {
         if (rc) return rc;
     }
     PassArgs a;
-    fill_args(ctx, a, 0);
+    fill_args(ctx, a, 0, ctx->n);
     size_t rs = ctx->prec == M2M_FP32C ? 4 : 8;
     size_t sm = rs * ((ctx->edge_len + 3) & ~3) + rs * ((ctx->prior.nE + 4) & ~3) + rs * ((ctx->prior.nL + 4) & ~3) + 16;
     int g = ctx->nsm * 4;
@@ -1899,6 +1900,7 @@ struct m2m_batch {
     std::vector<m2m_ctx *> ctx;
     cudaStream_t st = nullptr;
     bool fusable = false;        // one launch per stage is possible
+    long long n_all = 0;         // particles of all models: of a fused launch
     int layout = 0;
     int pk = 0;                  // common potential signature (PK_ANY if they differ)
     int period = 0;              // common moving-prior period (0: flat)
@@ -1956,7 +1958,7 @@ int batch_upload(m2m_batch *b) {
         int rc = finish_record(c);
         if (rc) return berr(b, rc, "model %d record: %s", m, c->err.c_str());
         c->stat_par = 0;
-        fill_args(c, pa[m], 0);
+        fill_args(c, pa[m], 0, b->n_all);
         pa[m].rec_chi_nblk = b->rcount[m];
         pa[m].rec_stat_nblk = b->pcount[m];
         pa[m].rec_ticket = c->d_rec_ticket + 1;
@@ -1993,7 +1995,7 @@ int batch_upload(m2m_batch *b) {
 
 size_t batch_smem(const m2m_batch *b, int flags) {
     size_t sm = 0;
-    for (m2m_ctx *c : b->ctx) sm = std::max(sm, pass_smem(c, flags));
+    for (m2m_ctx *c : b->ctx) sm = std::max(sm, pass_smem(c, flags, b->n_all));
     return sm;
 }
 
@@ -2217,9 +2219,7 @@ int m2m_batch_init(m2m_batch **out, int32_t precision, int32_t nmodels, const m2
         for (int k = 0; k < c->nsets; ++k)
             if (c->sets[k].psf_shift) b->fusable = false;   // seeing draws need each model's push count
     }
-    long long n_all = 0;
-    for (m2m_ctx *c : b->ctx) n_all += c->n;
-    for (m2m_ctx *c : b->ctx) c->launch_n = n_all;
+    for (m2m_ctx *c : b->ctx) b->n_all += c->n;
     if (b->fusable) {
         int rc = batch_plan(b, 1);
         if (rc) {
