@@ -1207,7 +1207,8 @@ __device__ __forceinline__ void gh_red_stream(float vlos, const float4 *r, float
     fx_red_fast(Lo, Mid, b + 4, Wg * fmaf(m2, fmaf(K4, m2, c.w), (c.w * c.w) * C4));
 }
 
-// (b: index of the lower parts, h: of the high part)
+// (b: index of the lower parts, hb: of the high part; V mod 2^32 wraps, so it is
+// formed unsigned)
 __device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, int hb, float v, float fscale, int sh,
                                        bool &ovf) {
     const float S = v * fscale;
@@ -1219,7 +1220,7 @@ __device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, int hb
         l = __float_as_int(r + FX_MAGIC) - 0x4B400000;
         const int A = (h + 32768) >> 16;
         const int mid = h - (A << 16);
-        atomicAdd(Lo + b, l + (int)((unsigned)mid << 16));
+        atomicAdd(Lo + b, (int)((unsigned)l + ((unsigned)mid << 16)));
         atomicAdd(Mid + b, mid);
         if (A) atomicAdd(Hi + hb, A);
     } else {
@@ -1227,7 +1228,7 @@ __device__ __forceinline__ void fx_red(int *Lo, int *Mid, int *Hi, int b, int hb
         const long long hh = (q + 32768) >> 16;
         const long long A = (hh + 32768) >> 16;
         const int mid = (int)(hh - (A << 16));
-        atomicAdd(Lo + b, (int)(q - (hh << 16)) + (int)((unsigned)mid << 16));
+        atomicAdd(Lo + b, (int)((unsigned)(q - (hh << 16)) + ((unsigned)mid << 16)));
         atomicAdd(Mid + b, mid);
         atomicAdd(Hi + hb, (int)A);
     }

@@ -512,7 +512,8 @@ __device__ __forceinline__ void fx_totals(const PassArgs &a, const PassSmem<floa
     const int R = S.hrep, o = lane >> 1;
     for (int k0 = 16 * w; k0 < nobs; k0 += 16 * nw) {
         const int k = k0 + o;
-        int lo = 0, mid = 0;
+        unsigned lo = 0u;                  // (wraps)
+        int mid = 0;
         if (k < nobs) {
             int off = 0, nmom = 1;
             for (int q = 0; q < a.nsets; ++q)
@@ -522,7 +523,7 @@ __device__ __forceinline__ void fx_totals(const PassArgs &a, const PassSmem<floa
 #pragma unroll 4
             for (int q = 0; q < (R >> 1); ++q) {
                 const int i = base + ((s + q) & (R - 1)) * nmom;
-                lo += S.hL[i];
+                lo += (unsigned)S.hL[i];
                 mid += S.hM[i];
                 if (clear) { S.hL[i] = 0; S.hM[i] = 0; }
             }
@@ -530,7 +531,7 @@ __device__ __forceinline__ void fx_totals(const PassArgs &a, const PassSmem<floa
         lo += __shfl_xor_sync(0xffffffffu, lo, 1);
         mid += __shfl_xor_sync(0xffffffffu, mid, 1);
         if (k < nobs && !(lane & 1)) {
-            const long long v = total(k, lo, mid);
+            const long long v = total(k, (int)lo, mid);
             if (clear) S.hH[k] = 0;
             f(k, v);
         }
