@@ -31,7 +31,9 @@
  *  - Host arrays passed in descriptors (edges, targets, GH parameters) are
  *    copied during the call; the caller may free them afterwards.
  *  - Scratch memory (partial histograms, cell tables) is library-owned,
- *    allocated in m2m_init and freed by m2m_free.
+ *    allocated in m2m_init and freed by m2m_free; m2m_velocity_moments
+ *    allocates its sums (32 bytes per shell) at the first call and where a
+ *    later one has more shells.
  *  - Errors found by kernels (non-finite weights, fixed-point overflow) are
  *    sticky and reported by the next m2m_get_* call.
  *  - Every scatter records each particle's cells (library-owned, 4 bytes per
@@ -44,6 +46,14 @@
  *    of evaluating the expansion again; a recompute of the expansion drops
  *    it.  A caller that changes x..z itself must call m2m_observe (which
  *    drops it too) before the next push.
+ *  - M2M_FP64 keeps 56 bytes per particle (library-owned) for m2m_step: what
+ *    a step computes and the next one of the same call needs again
+ *    (ln(w/w_hat) with the part its rounding left out, the force at the new
+ *    positions, the Gauss-Hermite factors).  Nothing is kept from one call to
+ *    the next.  They are allocated only where they are less than a quarter of
+ *    the device's free memory at m2m_init; without them each step computes
+ *    these values itself (more slowly; the results differ by the rounding of
+ *    the logarithm).  m2m_set_force_cache(ctx, 0) gives them back.
  *  - M2M_FP32C keeps ln w_hat_i per particle in float (library-owned, 4
  *    bytes per particle) for the weight update; it is taken from w_hat at
  *    m2m_init and rewritten with w_hat at every prior recompute.  A caller
@@ -435,7 +445,10 @@ int m2m_autotune(m2m_ctx *ctx, int32_t steps_per_trial, const char *cache_path, 
  * (default 1; see the conventions at the top): 0 evaluates the expansion
  * twice per push, at the old and at the new positions.  The kept force is
  * the same function of the same positions and node table, so the results
- * are bit-identical either way.  Applies from the next push. */
+ * are bit-identical either way.  Applies from the next push.
+ * M2M_FP64: also everything else m2m_step keeps between its steps (see the
+ * conventions); 0 waits for the stream and frees the memory, a later 1
+ * allocates it again by the rule of m2m_init. */
 int m2m_set_force_cache(m2m_ctx *ctx, int32_t enable);
 
 /* Persistent multi-step launches (on by default).  Where they apply -- an

@@ -691,6 +691,18 @@ void free_events(m2m_ctx *c) {
     c->ev_free.clear();
 }
 
+// FP64: the buffer of what a pass leaves for the next one, only where it
+// leaves the caller most of the memory (without it every pass computes these
+// values itself).
+void keep_alloc(m2m_ctx *c) {
+    if (c->prec != M2M_FP64) return;
+    size_t freeb = 0, totb = 0;
+    if (cudaMemGetInfo(&freeb, &totb) == cudaSuccess && C64_BYTES * (size_t)c->n < freeb / 4 &&
+        cudaMalloc((void **)&c->d_c64, C64_BYTES * (size_t)c->n) != cudaSuccess)
+        c->d_c64 = nullptr;
+    cudaGetLastError();
+}
+
 void free_all(m2m_ctx *c) {
     free_events(c);
     void *ptrs[] = {c->d_edges, c->d_gh, c->d_Y, c->d_sigma, c->d_isig, c->d_out, c->d_coef_d,
@@ -1089,15 +1101,7 @@ int m2m_init(m2m_ctx **ctx_out, int32_t precision, int64_t n, void *x, void *y, 
         ALLOC(ctx->d_cell_cnt, 4 * (size_t)ctx->ncells);
         ALLOC(ctx->d_cell_mean, 8 * (size_t)ctx->ncells);
     }
-    if (!f32) {
-        // only where it leaves the caller most of the memory; without it every
-        // pass computes these values itself
-        size_t freeb = 0, totb = 0;
-        if (cudaMemGetInfo(&freeb, &totb) == cudaSuccess && C64_BYTES * (size_t)n < freeb / 4 &&
-            cudaMalloc((void **)&ctx->d_c64, C64_BYTES * (size_t)n) != cudaSuccess)
-            ctx->d_c64 = nullptr;
-        cudaGetLastError();
-    }
+    keep_alloc(ctx);
 #undef ALLOC
 
     // tables: float edges are the smallest float >= the double edge
@@ -1835,6 +1839,12 @@ int m2m_set_force_cache(m2m_ctx *ctx, int32_t enable) {
     if (!ctx) return M2M_ERR_ARG;
     ctx->facc_off = enable == 0;
     ctx->facc_valid = false;
+    if (!enable && ctx->d_c64) {
+        CU(cudaStreamSynchronize(ctx->st));       // passes in flight use it
+        CU(cudaFree(ctx->d_c64));
+        ctx->d_c64 = nullptr;
+    }
+    if (enable && !ctx->d_c64) keep_alloc(ctx);
     return M2M_OK;
 }
 
