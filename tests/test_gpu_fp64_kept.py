@@ -27,10 +27,6 @@ def _targets(P):
     return P
 
 
-def _keep(ctx, on):
-    assert B.library().m2m_set_force_cache(ctx.ptr, int(on)) == 0
-
-
 # one call of 7 steps with the buffer and without it.  The force and the
 # Gauss-Hermite factors are the same functions of the same arguments; the
 # logarithm differs by its rounding and the sums by their order: the bounds of
@@ -44,7 +40,7 @@ def test_kept_and_computed_values_agree(name, n):
     out = []
     for on in (True, False):
         ctx = B.from_problem(P, "fp64")
-        _keep(ctx, on)
+        ctx.m2m_set_force_cache(on)
         ctx.m2m_step(7)
         y, _, Dt = ctx.m2m_get_obs()
         out.append(dict(ctx.state(), y_obs=y, Dt=Dt))
@@ -61,12 +57,12 @@ def test_memory_is_given_back_and_taken_again():
     n = 2_000_000
     ctx = B.from_problem(_targets(_problem("plain-fp64", n)), "fp64")
     for on in (True, False, True):                       # every kernel loaded
-        _keep(ctx, on)
+        ctx.m2m_set_force_cache(on)
         ctx.m2m_step(2)
     torch.cuda.synchronize()
     free = [torch.cuda.mem_get_info()[0]]
     for on in (False, True, True, False):
-        _keep(ctx, on)
+        ctx.m2m_set_force_cache(on)
         free.append(torch.cuda.mem_get_info()[0])
         ctx.m2m_step(2)
     ctx.m2m_free()
