@@ -1912,7 +1912,7 @@ struct m2m_batch {
     bool fusable = false;        // one launch per stage is possible
     long long n_all = 0;         // particles of all models: of a fused launch
     int layout = 0;
-    int pk = 0;                  // common potential signature (PK_ANY if they differ)
+    int pk = PK_ANY;             // common potential signature of the step at hand (PK_ANY if they differ)
     int period = 0;              // common moving-prior period (0: flat)
     PassArgs *d_pass = nullptr;  // per-model arguments
     ResArgs *d_res = nullptr;
@@ -1928,7 +1928,7 @@ struct m2m_batch {
     void *d_gather = nullptr;    // record gather: source pointers, records, error words
     long long t = 0;
     int last_mode = 0;
-    std::map<std::tuple<long long, long long, int>, cudaGraphExec_t> graphs;
+    std::map<std::tuple<long long, long long, int, int>, cudaGraphExec_t> graphs;
     std::string err;
 };
 
@@ -1973,6 +1973,7 @@ int batch_upload(m2m_batch *b) {
         pa[m].rec_stat_nblk = b->pcount[m];
         pa[m].rec_ticket = c->d_rec_ticket + 1;
         pa[m].rec_base = 0;
+        pa[m].fx_atomic = 1;                 // whatever the model's own passes do: the batched residual reads totals
         pa[m].epoch = 0;                     // unused: a fused batch has no seeing
         ResArgs &r = ra[m];
         memset(&r, 0, sizeof r);
@@ -2219,10 +2220,7 @@ int m2m_batch_init(m2m_batch **out, int32_t precision, int32_t nmodels, const m2
     m2m_ctx *c0 = b->ctx[0];
     b->fusable = precision == M2M_FP32C && c0->layout != 0;
     b->layout = c0->layout;
-    b->pk = potential_signature(c0);
     b->period = c0->prior.kind == M2M_PRIOR_FLAT ? 0 : c0->prior.period;
-    for (m2m_ctx *c : b->ctx)
-        if (potential_signature(c) != b->pk) b->pk = PK_ANY;
     for (m2m_ctx *c : b->ctx) {
         const int per = c->prior.kind == M2M_PRIOR_FLAT ? 0 : c->prior.period;
         if (c->layout != b->layout || per != b->period || c->sh_on) b->fusable = false;
@@ -2245,9 +2243,15 @@ int m2m_batch_init(m2m_batch **out, int32_t precision, int32_t nmodels, const m2
 int m2m_batch_step(m2m_batch *b, int64_t nsteps) {
     if (!b || nsteps < 0) return berr(b, M2M_ERR_ARG, "bad argument");
     if (nsteps == 0) return M2M_OK;
-    bool pending = false;
-    for (m2m_ctx *c : b->ctx) pending |= c->pending;
-    if (!b->fusable || pending) {
+    // (a model may have been given another layout or potential through its context)
+    bool single = !b->fusable;
+    int pk = potential_signature(b->ctx[0]);
+    for (m2m_ctx *c : b->ctx) {
+        single |= c->pending || c->layout != b->layout || c->sh_on;
+        if (potential_signature(c) != pk) pk = PK_ANY;
+    }
+    b->pk = pk;
+    if (single) {
         for (int m = 0; m < b->nmodels; ++m) {
             int rc = m2m_step(b->ctx[m], nsteps);
             if (rc) return berr(b, rc, "model %d: %s", m, b->ctx[m]->err.c_str());
@@ -2277,10 +2281,10 @@ int m2m_batch_step(m2m_batch *b, int64_t nsteps) {
     b->up_step = -1;
     if (e != cudaSuccess) return berr(b, M2M_ERR_CUDA, "step counter: %s", cudaGetErrorString(e));
     const bool graphable = b->st != nullptr && b->st != cudaStreamLegacy && b->st != cudaStreamPerThread;
-    // (the launches of a graph keep their shared memory size, which follows the
-    // models' histogram copies)
+    // (the launches of a graph keep their kernel, which follows the potentials,
+    // and their shared memory size, which follows the models' histogram copies)
     const auto key = std::make_tuple((long long)nsteps, b->period ? t0 % b->period : 0ll,
-                                     (int)batch_smem(b, F_STEADY | F_MINMAX));
+                                     (int)batch_smem(b, F_STEADY | F_MINMAX), b->pk);
     bool launched = false;
     if (graphable) {
         auto it = b->graphs.find(key);
