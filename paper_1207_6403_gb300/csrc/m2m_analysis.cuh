@@ -47,7 +47,7 @@ inline int vmoments_copies(int nsh) {
 // reciprocal of r^2 R^2 and no square root.  Bound by the FP64 pipe (one warp
 // instruction in 16 cycles per SM): 31 of them per particle, against about
 // 100 and the serialised adds before (1M particles, 8 shells: the call took
-// 576 us, now 92 us).
+// 576 us, now 71 us).
 template <class R>
 __global__ void __launch_bounds__(256) k_vmoments(const R *x, const R *y, const R *z, const R *vx, const R *vy,
                                                   const R *vz, const double *w, long long n, const R *e2,

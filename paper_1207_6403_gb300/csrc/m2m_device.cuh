@@ -80,10 +80,10 @@ struct PassArgs {
     const void *edge_tab; int edge_len;     // R
     const void *gh_tab;   int gh_len;       // R, 5 per GH cell: V, 1/S, c1, t2, norm
     const void *coef;                       // R[nobs]
-    void *slots;                            // FP64: [grid][nobs] double per-block sums
-    unsigned long long *y_acc;              // FP32C: [nobs] int64 fixed-point totals
+    void *slots;                            // FP32C without atomics: [grid][nobs] int64 per-block sums
+    unsigned long long *y_acc;              // [nobs] totals: int64 fixed point (FP32C) or double
     int fx_atomic;                          // FP32C: flush to y_acc with atomics (else slots)
-    int hrep;                               // FP32C: copies of the block histogram's lower parts (see hist_copies)
+    int hrep;                               // copies of the block histogram (FP32C: of its lower parts; see hist_copies)
     int fx_shift;                           // fixed point: value * 2^fx_shift
     int cell_shift;                         // FP32C prior-cell sums: weight * 2^cell_shift
     double *stat_slots;                     // [grid][2]: S, sum w
@@ -98,7 +98,7 @@ struct PassArgs {
     double *c64_m, *c64_g;                  // m and the Gaussian factor of the GH cell
     int c64_read;
     const double *exp_tab;                  // FP64: 2^(j/128)
-    void *facc; int facc_read;              // expansion potentials: force at the positions (R, [3][n]) or NULL
+    void *facc; int facc_read;              // force at the positions (R, [3][n]; see kdk) or NULL
     // record of the preceding step, left by its residual to this pass (the
     // first block to finish its particles writes it; see record_warp)
     // (rec_pending REC_EVERY: each launch of nblk tickets has a record to write)

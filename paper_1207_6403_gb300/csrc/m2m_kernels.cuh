@@ -1216,14 +1216,6 @@ __device__ __forceinline__ void residual_obs(const ResArgs &a, int j, double yv,
 
 #ifdef M2M_COMMON_KERNELS
 
-// Deterministic strided sum over the block: thread k adds k, k+NT, ... in
-// order, then a fixed shuffle tree.
-__device__ __forceinline__ double block_sum_strided(const double *v, int stride, int off, int cnt, double *red) {
-    double s = 0.0;
-    for (int k = threadIdx.x; k < cnt; k += blockDim.x) s += v[(long long)k * stride + off];
-    return block_sum(s, red);
-}
-
 // Totals (fx_atomic): one thread per observable in small blocks; the totals
 // are already summed by the pass's atomics, exact integers in FP32C and
 // doubles in FP64 (re-zeroed here for the next scatter; reducing FP64 slots

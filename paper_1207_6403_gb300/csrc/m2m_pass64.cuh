@@ -2,7 +2,7 @@
 //
 // An FP64 warp instruction takes 16 cycles of an SM here (an FP32 one a
 // quarter of a cycle), so the pass is bound by the number of double
-// operations per particle, not by memory (120 of 190 bytes moved are the
+// operations per particle, not by memory (120 of 200 to 240 bytes moved are the
 // step's own and take a twentieth of the time).  What follows from that:
 //  - inside one m2m_step call a pass leaves what the next one would compute
 //    again from the same particle: the force at the new position, ln(w/w_hat)
@@ -26,7 +26,7 @@
 //  - warps are dealt chunks of 32 particles round the blocks, so that a small
 //    model occupies every SM.
 // 300,000 particles, pixels + apertures in the logarithmic potential: a step
-// takes 109 us, 454 before; 20,000 particles, shells + annuli, 21 us, 125
+// takes 111 us, 454 before; 20,000 particles, shells + annuli, 21 us, 125
 // before.  Global double atomics instead of the shared histogram were slower
 // (300,000 particles 139 us a step, shells + annuli at 200,000 276 against 79:
 // many particles share a total).
@@ -144,9 +144,9 @@ __device__ __forceinline__ bool mid_weight(double w) {
 // longer moves (|d| below half an ulp) would leave the sum moving on.  As it
 // is, the error after 4000 steps is that of one fresh logarithm (rms 6e-17;
 // L + d alone 5e-15 and more).  Seven FP64 operations, where the quotient and
-// the logarithm take 40: 300,000 particles, pixels + apertures, 25 steps 2820
-// us; with the series and so the carry only below |d| = 2^-10, where half of
-// the warps have a lane beyond it, 3210.
+// the logarithm take 40: where half of the warps took those (a series and so
+// the carry only below |d| = 2^-10), 300,000 particles, pixels + apertures, 25
+// steps took 3210 us against 2820.
 __device__ __forceinline__ double log_carry(double L, double &l, double w, double wn, double d, double e) {
     const double rem = fma(w, e, w - wn);            // the difference is exact (|e| < 2^-4)
     double y;
