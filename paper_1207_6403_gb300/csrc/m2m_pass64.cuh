@@ -16,7 +16,8 @@
 //  - an expansion's force is a call (m2m_device.cuh, ex_accel_call);
 //  - exp is table driven (P. T. P. Tang, ACM TOMS 15 (1989) 144: exp(x) =
 //    2^(k/128) exp(r), |r| <= ln 2/256, a quintic in r), 10 operations; the
-//    weight's exp(d) is 1 + its series to d^8 for |d| < 2^-5 (the rest is below 2^-63);
+//    weight's exp(d) is 1 + its series, to d^5 for |d| < 2^-10 and to d^8 for
+//    |d| < 2^-5 (what is left out is below 2^-58 of d);
 //  - the moments are polynomials of m with the constants of gh_record, no
 //    division;
 //  - a double shared-memory add is a compare-and-swap loop, which the lanes
@@ -151,7 +152,7 @@ __device__ __forceinline__ double log_carry(double L, double &l, double w, doubl
     const double rem = fma(w, e, w - wn);            // the difference is exact (|e| < 2^-4)
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(wn));               // 20 bits: rem is below an ulp
-    const double c = d + (l - rem * y);
+    const double c = d + fma(-rem, y, l);
     const bool first = ((unsigned)__double2hiint(L) & 0x7fffffffu) >= ((unsigned)__double2hiint(c) & 0x7fffffffu);
     const double p = first ? L : c, q = first ? c : L, s = p + q;
     l = q - (s - p);
@@ -304,12 +305,15 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
                     }
                     const double G = a.mu * (-Lw - a.ent_c) - dot;
                     const double d = a.eps_dt * G;
-                    const bool small = ((unsigned)__double2hiint(d) & 0x7fffffffu) < 0x3FA00000u;   // |d| < 2^-5
+                    const unsigned dx = (unsigned)__double2hiint(d) & 0x7fffffffu;
                     double e = 0.0;
-                    if (small) {
-                        e = fma(d, 1.0 / 40320.0, 1.0 / 5040.0);
-                        e = fma(d, e, 1.0 / 720.0);
-                        e = fma(d, e, 1.0 / 120.0);
+                    if (dx < 0x3FA00000u) {                      // |d| < 2^-5
+                        e = 1.0 / 120.0;
+                        if (dx >= 0x3F500000u) {                 // |d| >= 2^-10
+                            e = fma(d, 1.0 / 40320.0, 1.0 / 5040.0);
+                            e = fma(d, e, 1.0 / 720.0);
+                            e = fma(d, e, 1.0 / 120.0);
+                        }
                         e = fma(d, e, 1.0 / 24.0);
                         e = fma(d, e, 1.0 / 6.0);
                         e = fma(d, e, 0.5);
@@ -320,9 +324,12 @@ __device__ __forceinline__ void pass64_body(const PassArgs &a, const int bid, co
                         wn = w * exp(d);
                     }
                     wr = wn;
-                    if (a.c64_lnw && small && mid_weight(wn)) Lk = log_carry(Lw, Ll, w, wn, d, e);
-                    else if (a.c64_lnw) { Lk = log(wn / a.what[i]); Ll = 0.0; }
-                    Lw = Lw + d;
+                    if (a.c64_lnw && dx < 0x3FA00000u && mid_weight(wn)) {
+                        Lk = Lw = log_carry(Lw, Ll, w, wn, d, e);
+                    } else {
+                        if (a.c64_lnw) { Lk = log(wn / a.what[i]); Ll = 0.0; }
+                        Lw = Lw + d;
+                    }
                     if (d_bad(wn)) bad = true;
                 }
                 if (fl & F_STATS) {
