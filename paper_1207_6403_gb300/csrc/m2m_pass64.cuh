@@ -27,7 +27,7 @@
 //  - warps are dealt chunks of 32 particles round the blocks, so that a small
 //    model occupies every SM.
 // 300,000 particles, pixels + apertures in the logarithmic potential: a step
-// takes 111 us, 454 before; 20,000 particles, shells + annuli, 21 us, 125
+// takes 111 us, 454 before; 20,000 particles, shells + annuli, 22 us, 125
 // before.  Global double atomics instead of the shared histogram were slower
 // (300,000 particles 139 us a step, shells + annuli at 200,000 276 against 79:
 // many particles share a total).
