@@ -506,10 +506,11 @@ int m2m_get_timing(m2m_ctx *ctx, m2m_timing *out);
  * precision, the other step parameters and the stream.  When every model
  * is FP32C with the same compiled observable layout and the same prior
  * schedule, one kernel launch advances all models' particles per stage
- * (blocks shared out in proportion to N) and, on a non-default stream, the
- * launch sequence of m2m_batch_step is captured once into a CUDA graph and
- * replayed; otherwise the models are stepped one after another.  Results
- * are those of stepping each model alone. */
+ * (blocks of equal work) and, on a non-default stream, the launch sequence
+ * of m2m_batch_step is captured once into a CUDA graph and replayed;
+ * otherwise, and while a model has been given another layout or an expansion
+ * potential through its context, the models are stepped one after another.
+ * Results are those of stepping each model alone. */
 typedef struct {
     int64_t n;
     void *x, *y, *z, *vx, *vy, *vz;   /* device, caller-owned (as m2m_init) */
